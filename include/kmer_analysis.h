@@ -136,8 +136,9 @@ typedef struct {
  * survivors come out grouped by partition.  With it, query, query_into and
  * merge_contigs leave them sorted by key (word 0 first, numerically; the
  * same as the lexicographic order of the k-mers) with count, ext and cls
- * moved along: a least-significant-digit radix sort on the device, 2k/8
- * passes over the keys, in place in the result arrays.  Its scratch (about
+ * moved along: a sample sort on the device (above 2^28 survivors, or when
+ * thousands of k-mers begin with the same 32 bases, a radix sort of 2k/8
+ * passes over the keys), in place in the result arrays.  Its scratch (about
  * 8W + 74 bytes per survivor) reuses the query's record buffers when they are
  * large enough.  query_into with page-locked host arrays (KMER_HOST) then
  * stages through the analysis's device buffers as with KMER_HOST_STAGED.

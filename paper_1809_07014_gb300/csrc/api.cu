@@ -1017,7 +1017,7 @@ int sort_results(kmer_analysis* h) {
     if (!(h->p.flags & KMER_FLAG_SORTED_OUTPUT) || h->n_out < 2) return KMER_OK;
     if (h->n_out >= 0xFFFFFFFFull) return fail(KMER_ERR_INVALID_ARG, "sorted output limited to 2^32 - 2 survivors");
     const unsigned W = h->W();
-    const size_t need = sort_scratch_bytes(W, h->n_out);
+    const size_t need = sort_scratch_bytes(W, h->n_out, h->res_windows, h->num_sms);
     void* scratch = nullptr;
     for (DevBuf* b : {&h->l2_rec, &h->l1_rec, &h->hbm})
         if (!scratch && b->p && b->bytes >= need) scratch = b->p;
@@ -1029,13 +1029,22 @@ int sort_results(kmer_analysis* h) {
     CK(cudaMemsetAsync(&m->status, 0, sizeof m->status, h->stream));
     TRY(prof_begin(h, kmer_analysis::STG_SORT));
     unsigned launches = 0;
-    CK(launch_sort_survivors(W, h->res_keys, h->res_count, h->res_ext, h->res_cls, h->n_out, h->p.k, scratch,
-                             &m->status, h->num_sms, &launches, h->stream));
+    CK(launch_sort_survivors(W, h->res_keys, h->res_count, h->res_ext, h->res_cls, h->n_out, h->res_windows, h->p.k,
+                             scratch, &m->status, h->num_sms, &launches, h->stream));
     TRY(prof_end(h, kmer_analysis::STG_SORT));
-    h->st.launches += launches;
     h->lk_cap = 0;  // positions changed
     TRY(read_misc(h));
     TRY(prof_collect(h));
+    if (h->host_misc->status & ST_SORT_SPLIT) {  // thousands of keys alike in their first 64 bits
+        CK(cudaMemsetAsync(&m->status, 0, sizeof m->status, h->stream));
+        TRY(prof_begin(h, kmer_analysis::STG_SORT));
+        CK(launch_sort_by_digits(W, h->res_keys, h->res_count, h->res_ext, h->res_cls, h->n_out, h->p.k, scratch,
+                                 &m->status, h->num_sms, &launches, h->stream));
+        TRY(prof_end(h, kmer_analysis::STG_SORT));
+        TRY(read_misc(h));
+        TRY(prof_collect(h));
+    }
+    h->st.launches += launches;
     if (h->host_misc->status & ST_TIMEOUT) return fail(KMER_ERR_TIMEOUT, "the sort's look-back gave up");
     if (h->host_misc->status & ST_SORT_RANGE) return fail(KMER_ERR_CUDA, "internal: sort position out of range");
     return KMER_OK;

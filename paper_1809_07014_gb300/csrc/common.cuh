@@ -45,6 +45,7 @@ enum StatusBits : unsigned int {
     ST_COUNTER_OVERFLOW = 1u << 6,
     ST_L2_PLAN = 1u << 7,        // the level-2 planner found the leaf layout larger than the buffer
     ST_SORT_RANGE = 1u << 8,     // a radix-sort position fell outside the survivors (write skipped)
+    ST_SORT_SPLIT = 1u << 9,     // a bucket of the sample sort is larger than one CTA sorts (nothing moved)
 };
 
 // Extension code of one window: left and right in {0 = none, 1..4 = A,C,G,T + 1},

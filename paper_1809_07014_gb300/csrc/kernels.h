@@ -94,15 +94,23 @@ cudaError_t launch_traverse_write(unsigned W, const unsigned long long* keys, co
                                   unsigned long long n, unsigned k, unsigned long long n_contigs, void* scratch,
                                   char* out, unsigned long long* contig_off, int num_sms, cudaStream_t s);
 
-// Survivors in ascending key order: LSD radix sort of the n keys (8-bit
-// digits over the 2k key bits, one-sweep passes, n < 2^32), then count / ext /
-// cls gathered through the permutation; all four arrays are rewritten in
-// place.  scratch: sort_scratch_bytes; *launches counts the kernels; status
-// gets ST_TIMEOUT if a look-back gave up and ST_SORT_RANGE if a position fell
-// outside [0, n) (its write skipped).  Synchronises the stream once (to skip
-// passes whose digit is constant).
-size_t sort_scratch_bytes(unsigned W, unsigned long long n);
+// Survivors in ascending key order (sort.cu): the n keys (n < 2^32, distinct),
+// count / ext / cls moved along, all four arrays rewritten in place.
+// `windows`: at least the sum of the counts.  scratch: sort_scratch_bytes;
+// *launches counts the kernels.  launch_sort_survivors is a sample sort up to
+// 2^28 survivors (above them the sort by digits); it sets ST_SORT_SPLIT in
+// *status, leaving the arrays as they were, when a bucket came out larger than
+// one CTA sorts (thousands of keys with the same first 64 bits): the caller
+// then calls launch_sort_by_digits, an LSD radix sort (8-bit digits over the
+// 2k key bits, one-sweep passes) that sets ST_TIMEOUT if a look-back gave up
+// and synchronises the stream once (to skip passes whose digit is constant).
+// Either sets ST_SORT_RANGE if a position fell outside its array (its write
+// skipped).
+size_t sort_scratch_bytes(unsigned W, unsigned long long n, unsigned long long windows, int num_sms);
 cudaError_t launch_sort_survivors(unsigned W, unsigned long long* keys, unsigned* count, unsigned* ext,
+                                  unsigned char* cls, unsigned long long n, unsigned long long windows, unsigned k,
+                                  void* scratch, unsigned* status, int num_sms, unsigned* launches, cudaStream_t s);
+cudaError_t launch_sort_by_digits(unsigned W, unsigned long long* keys, unsigned* count, unsigned* ext,
                                   unsigned char* cls, unsigned long long n, unsigned k, void* scratch,
                                   unsigned* status, int num_sms, unsigned* launches, cudaStream_t s);
 
