@@ -114,11 +114,13 @@ Geometry plan_geometry(unsigned k, unsigned long long windows, unsigned long lon
     g.W = (2 * k + 63) / 64;
     g.hb = 2 * k - 64 * (g.W - 1);
     g.bt = g.W == 1 ? 2 * k : 64;
-    // up to 0.7 of a leaf table of (estimated) distinct keys per leaf: the
-    // estimate carries a 15 % margin, so leaves hold about 0.3-0.6 of a table
-    // (fewer, fuller leaves amortise each leaf's sweep and barriers; a leaf
-    // that overflows is counted again in key ranges)
-    const unsigned long long target = std::max(64ull, (unsigned long long)cap_max * 7 / 10);
+    // up to 0.75 of a leaf table of (estimated) distinct keys per leaf: the
+    // estimate carries a 7 % margin, so leaves hold about 0.35-0.7 of a table
+    // (fewer, fuller leaves amortise each leaf's sweep and barriers: 300 M bases
+    // at k = 99 take 4.09 ms in leaves of 0.66 and 4.71 in leaves of 0.33; past
+    // 0.8 probes grow long, and a leaf that overflows is counted again in key
+    // ranges)
+    const unsigned long long target = std::max(64ull, (unsigned long long)cap_max * 3 / 4);
     unsigned p = leaf_bits ? leaf_bits : ceil_log2((basis + target - 1) / target);
     const unsigned need = g.bt > 58 ? g.bt - 58 : 0;  // partition bits implied by the record format
     p = std::max(p, need);
@@ -444,7 +446,7 @@ Plan make_plan(const kmer_analysis* h, unsigned long long windows, size_t budget
     if (gated_distinct) basis = std::min<unsigned long long>(windows, gated_distinct + gated_distinct / 8 + 1024);
     else if (h->p.distinct_hint) basis = std::min<unsigned long long>(h->p.distinct_hint, windows);
     else if (h->hist_k == h->p.k && h->hist_ratio > 0.0)  // learned from the previous query at this k
-        basis = std::min<unsigned long long>(windows, (unsigned long long)(1.15 * h->hist_ratio * (double)windows) + 1);
+        basis = std::min<unsigned long long>(windows, (unsigned long long)(1.07 * h->hist_ratio * (double)windows) + 1);
     pl.g = plan_geometry(h->p.k, windows, basis, budget, cap_max, h->p.leaf_bits, h->p.l1_bits, true, l1_slack(h));
     pl.passes = 1u << pl.g.ps;
     pl.budget = budget;

@@ -9,17 +9,28 @@
 // batch of the next leaf's records is already loading into registers.
 //
 // Table (shared memory, planes of `cap_max` entries, a leaf uses the first
-// `cap` slots): the tail word of each slot (0 = empty; record tail with the
-// extension bits replaced by a mark bit; bit 0 = being published, W > 2
-// only), W-1 head words (two-word keys keep tail and head side by side, one
-// 16-byte pair per slot claimed by a 128-bit CAS, in probe groups of two
-// slots), and nine 16-bit tallies packed in five 32-bit planes:
-// left A, C, G, T, "no left extension" (so that count = sum of the five left
-// lanes and needs no counter of its own), right A, C, G, T.  Slots are probed
-// in groups of 32 bytes of keys (one read compares four tails, or two
-// two-word keys).  A leaf with 65536 records or more (where a 16-bit tally
-// could wrap) is recounted exactly by the HBM-table fallback; one whose keys
-// do not fit its table is counted again in key ranges (leaf_split_kernel).
+// `cap` slots): the tail word of each slot (0 = empty; else the tail of the
+// record that claimed the slot, plus one: its key and that record's extension
+// code), W-1 head words (two-word keys keep tail and head side by side, one
+// 16-byte pair per slot claimed by a 128-bit CAS), and nine 16-bit tallies of
+// the other records, packed in five 32-bit planes: left A, C, G, T, "no left
+// extension" (so that count = one + the five left lanes and needs no counter
+// of its own), right A, C, G, T.  Slots are probed in groups of 16 bytes of
+// keys (two tails, or one two-word key), a key's groups a hashed step apart.
+// A leaf with 65536 records or more (where a 16-bit tally could wrap) is
+// recounted exactly by the HBM-table fallback; one whose keys do not fit its
+// table is counted again in key ranges (leaf_split_kernel).
+//
+// What bounds it: latency of the probe rounds and the issue slots (about 0.67
+// instructions a cycle and scheduler, half of the shared-memory pipe), not
+// DRAM.  On the 2-Gbase reads at k = 31 (1.6 G records, 508 M keys) 18.5 ->
+// 14.4 ms, at k = 99 (103 M records, 89 M keys) 5.3 -> 3.7 ms, from: the
+// claiming record keeping its extension code in the slot (no tally for a third
+// of the records at k = 31, for six in seven at k = 99; most k-mers are seen
+// once), hashed steps between groups (consecutive groups clustered: leaves
+// above 0.6 of a table overflowed their probe limit), 32-bit shared-memory
+// addresses, job fields in shared memory instead of global loads in the sweep,
+// four slots per lane in the sweep, and fuller leaves (0.75 of a table).
 //
 // Every plane is zero between leaves: the sweep clears each slot after
 // reading it, so no separate clearing pass is needed.
@@ -32,13 +43,14 @@ constexpr int kLeafThreads = 512;
 constexpr int kLeafWarps = kLeafThreads / 32;
 constexpr unsigned kLeafFull = 1u, kLeafTimeout = 4u;
 constexpr unsigned kSpinLimit = 1u << 22;
-constexpr unsigned kMaxGroupProbes = 16;  // 64 slots; a longer chain sends the leaf to the fallback
+constexpr unsigned kMaxRounds = 64;       // probe rounds of one record; past them the leaf goes to its key ranges
 constexpr unsigned kLanePlanes = 5;
 constexpr unsigned kMaxSubBits = 4;       // a leaf is split into at most 16 key ranges
-// Slot tail of an occupied key: the record tail with its extension bits
-// replaced by this mark; bit 0 marks a slot being published (W > 2).
-constexpr unsigned long long kKeyMark = 32ull;
-constexpr unsigned long long kBusy = 1ull;
+// Slot tail of an occupied key: the tail of the record that claimed it plus
+// one, so that its low six bits hold that record's extension code + 1 (at most
+// 37, never 0; 0 = empty slot).  The claiming record needs no tally of its own.
+// kBusy in those bits marks a slot being published (W > 2).
+constexpr unsigned kBusy = 63u;
 
 template <int W>
 struct LeafShape {
@@ -91,68 +103,66 @@ __device__ __forceinline__ LeafInfo leaf_info(const Job& j, unsigned leaf) {
 }
 
 template <int W>
-__device__ __forceinline__ void load_batch(const LeafInfo& li, unsigned long long first,
+__device__ __forceinline__ void load_batch(const LeafInfo& li, unsigned first,
                                            unsigned long long (&r)[LeafShape<W>::U][W]) {
     constexpr int U = LeafShape<W>::U;
     const unsigned long long* src = li.recs + li.start * W;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const unsigned long long i = first + (unsigned long long)u * kLeafThreads + threadIdx.x;
+        const unsigned i = first + u * kLeafThreads + threadIdx.x;
 #pragma unroll
-        for (int w = 0; w < W; ++w) r[u][w] = (li.ok && i < li.n) ? __ldcs(src + i * W + w) : 0ull;
+        for (int w = 0; w < W; ++w) r[u][w] = (li.ok && i < li.n) ? __ldcs(src + (size_t)i * W + w) : 0ull;
     }
 }
 
+// The table's planes as 32-bit shared-memory addresses (bytes): every access
+// below is an explicit shared-memory instruction with a 32-bit address, so no
+// address is computed in 64 bits.
 struct Table {
-    unsigned long long* tail;   // [cap_max]
-    unsigned long long* heads;  // [(W-1) * cap_max]
-    unsigned* lanes;            // [5 * cap_max]
-    unsigned* list;             // [cap_max]
-    unsigned stride;            // cap_max
+    unsigned tail;    // 8 bytes a slot (two-word keys: 16, tail and head)
+    unsigned heads;   // W - 1 planes of 8 bytes a slot
+    unsigned lanes;   // 5 planes of 4 bytes a slot
+    unsigned list;    // 4 bytes a slot
+    unsigned stride;  // slots of a plane
 };
 
-// Two adjacent slots' tail words, re-read from shared memory on every call.
-__device__ __forceinline__ ulonglong2 lds_v2_volatile(const unsigned long long* p) {
-    ulonglong2 r;
-    asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];"
-                 : "=l"(r.x), "=l"(r.y)
-                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+__device__ __forceinline__ unsigned lds32(unsigned a) {
+    unsigned v;
+    asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long lds64(unsigned a) {
+    unsigned long long v;
+    asm volatile("ld.volatile.shared.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 lds128(unsigned a) {
+    uint4 r;
+    asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(a) : "memory");
     return r;
 }
-
-// Lane q in 0..8 lives in plane q >> 1, half q & 1.
-__device__ __forceinline__ void bump(const Table& t, unsigned slot, unsigned q) {
-    atomicAdd(&t.lanes[(q >> 1) * t.stride + slot], 1u << (16 * (q & 1)));
+__device__ __forceinline__ void sts32(unsigned a, unsigned v) {
+    asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
-
-// Key words of a slot.  One-word keys: the tail plane.  Two-word keys:
-// (tail, head) pairs, 16 bytes per slot over the first two planes, claimed
-// whole by one 128-bit CAS.  Wider keys: the tail plane and W-1 head planes,
-// published with a busy bit.
-template <int W>
-__device__ __forceinline__ unsigned long long& slot_tail(const Table& t, unsigned s) {
-    return t.tail[W == 2 ? 2 * s : s];
+__device__ __forceinline__ void sts64(unsigned a, unsigned long long v) {
+    asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
 }
-template <int W>
-__device__ __forceinline__ unsigned long long slot_head(const Table& t, unsigned w, unsigned s) {
-    return W == 2 ? t.tail[2 * s + 1] : t.heads[(size_t)w * t.stride + s];
+__device__ __forceinline__ void sts128_zero(unsigned a) {
+    asm volatile("st.volatile.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(a), "r"(0u) : "memory");
 }
-template <int W>
-__device__ __forceinline__ void clear_key(const Table& t, unsigned s) {
-    if (W == 2) {
-        *reinterpret_cast<ulonglong2*>(t.tail + 2 * s) = make_ulonglong2(0ull, 0ull);
-    } else {
-        t.tail[s] = 0ull;  // head words of an empty slot are never read
-    }
+__device__ __forceinline__ void add_shared(unsigned a, unsigned v) {
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
-// Probe groups of a table of `cap` slots: 32 bytes of keys each.
-template <int W>
-__device__ __forceinline__ unsigned groups_of(unsigned cap) { return W == 2 ? cap / 2 : cap / 4; }
-
-// 128-bit compare-and-swap on shared memory: {lo, hi} replaces {0, 0};
-// returns the previous contents.
-__device__ __forceinline__ void cas128_shared(unsigned long long* p, unsigned long long lo, unsigned long long hi,
-                                              unsigned long long& old_lo, unsigned long long& old_hi) {
+// v replaces 0; returns the previous contents.
+__device__ __forceinline__ unsigned long long claim64(unsigned a, unsigned long long v) {
+    unsigned long long old;
+    asm volatile("atom.shared.cas.b64 %0, [%1], %2, %3;" : "=l"(old) : "r"(a), "l"(0ull), "l"(v) : "memory");
+    return old;
+}
+// {lo, hi} replaces {0, 0}; returns the previous contents.
+__device__ __forceinline__ void claim128(unsigned a, unsigned long long lo, unsigned long long hi,
+                                         unsigned long long& old_lo, unsigned long long& old_hi) {
     asm volatile(
         "{\n\t.reg .b128 cmp, val, old;\n\t"
         "mov.b128 cmp, {%4, %4};\n\t"
@@ -160,170 +170,266 @@ __device__ __forceinline__ void cas128_shared(unsigned long long* p, unsigned lo
         "atom.shared.cas.b128 old, [%5], cmp, val;\n\t"
         "mov.b128 {%0, %1}, old;\n\t}"
         : "=l"(old_lo), "=l"(old_hi)
-        : "l"(lo), "l"(hi), "l"(0ull), "r"((unsigned)__cvta_generic_to_shared(p))
+        : "l"(lo), "l"(hi), "l"(0ull), "r"(a)
         : "memory");
 }
 
-// Two-word keys: probe groups of two 16-byte slots.  A claim writes both
-// words at once, but a plain 16-byte read may still see a slot being
-// claimed with its tail and not yet its head; a tail match with another head
-// is read again atomically (a CAS that can only fail) before it counts as a
-// different key.
-__device__ __forceinline__ int find_slot2(const Table& t, const unsigned long long ktail,
-                                          const unsigned long long head, unsigned g, unsigned ngroups) {
-    for (unsigned probe = 0; probe < 2 * kMaxGroupProbes; ++probe) {
-        unsigned long long* grp = t.tail + 4 * g;
-        const ulonglong2 a = lds_v2_volatile(grp);
-        const ulonglong2 b = lds_v2_volatile(grp + 2);
+// Tally lane q in 0..8 of a slot lives in plane q >> 1, half q & 1.
+__device__ __forceinline__ void bump(const Table& t, unsigned slot, unsigned q) {
+    add_shared(t.lanes + 4 * ((q >> 1) * t.stride + slot), q & 1u ? 0x10000u : 1u);
+}
+
+// Key words of a slot.  One-word keys: the tail plane.  Two-word keys:
+// (tail, head) pairs, 16 bytes per slot over the first two planes, claimed
+// whole by one 128-bit CAS.  Wider keys: the tail plane and W-1 head planes,
+// published with a busy mark.
+template <int W>
+__device__ __forceinline__ unsigned long long slot_tail(const Table& t, unsigned s) {
+    return lds64(t.tail + (W == 2 ? 16 : 8) * s);
+}
+template <int W>
+__device__ __forceinline__ unsigned head_addr(const Table& t, unsigned w, unsigned s) {
+    return W == 2 ? t.tail + 16 * s + 8 : t.heads + 8 * (w * t.stride + s);
+}
+// Probe groups of a table of `cap` slots: 16 bytes of keys each (two tails, or
+// one two-word key), read by one shared-memory load.
+template <int W>
+__device__ __forceinline__ unsigned groups_of(unsigned cap) { return W == 2 ? cap : cap / 2; }
+
+// A tail (lo, hi words) of an occupied slot is the key of tail k (the low six
+// bits are the claiming record's extension code).
+__device__ __forceinline__ bool same_tail(unsigned lo, unsigned hi, unsigned klo, unsigned khi) {
+    return (((lo ^ klo) & ~63u) | (hi ^ khi)) == 0u && lo != 0u;
+}
+
+// Slot of a record's key, or kClaimed when the record claimed a new one,
+// kNoSlot after kMaxRounds full groups, kGaveUp after a wait that gave up.
+//
+// A key goes through groups home, home + step, ... of the table.  The slots of
+// a group fill in order and none empties while a leaf is counted, so a group's
+// first empty slot is the number of occupied ones, and a claim there can only
+// succeed when every slot before it holds a key that was compared: a key never
+// gets two slots.  Each round of the loop is one 16-byte load and at most one
+// claim.
+//
+// A lane leaves as soon as its record is settled and goes on to its next one
+// by itself.  The lanes of a warp drift apart that way, which pays: rounds are
+// latency (a load, a compare, a CAS), and lanes apart overlap theirs.
+constexpr int kClaimed = -1, kNoSlot = -2, kGaveUp = -3;
+
+template <int W>
+__device__ __forceinline__ int find_slot(const Table& t, const unsigned long long (&rec)[W], unsigned ngroups) {
+    constexpr unsigned GS = W == 2 ? 1 : 2;  // slots of a group
+    // home group from every in-leaf bit of z (the low bits of z depend on few
+    // bits of the key, its top bits are the leaf's): a multiplicative hash
+    const unsigned lo = (unsigned)rec[W - 1], khi = (unsigned)(rec[W - 1] >> 32), klo = lo + 1u;
+    const unsigned hsh = (lo & ~63u) * 0x9E3779B1u + khi * 0x85EBCA77u;
+    const unsigned long long ktail = rec[W - 1] + 1ull;
+    unsigned g = __umulhi(hsh, ngroups);
+    for (unsigned it = 0; it < kMaxRounds;) {
+        const unsigned ga = t.tail + 16 * g;
+        const uint4 a = lds128(ga);
+        if constexpr (W == 2) {
+            unsigned long long ct = (unsigned long long)a.y << 32 | a.x, ch = (unsigned long long)a.w << 32 | a.z;
+            if (a.x == 0u) {  // empty, or still being claimed
+                claim128(ga, ktail, rec[0], ct, ch);
+                if (ct == 0ull && ch == 0ull) return kClaimed;
+            }
+            if (same_tail((unsigned)ct, (unsigned)(ct >> 32), klo, khi)) {
+                // a plain read may catch a claim half done (the tail without its head):
+                // another head is read again by a CAS that cannot change the slot
+                if (ch != rec[0]) claim128(ga, 0ull, 0ull, ct, ch);
+                if (ch == rec[0]) return (int)g;
+            }
+        } else {
+            const unsigned occ = (a.x ? 1u : 0u) + (a.z ? 1u : 0u);
+            for (unsigned s = 0; s < occ; ++s) {
+                if (!same_tail(s ? a.z : a.x, s ? a.w : a.y, klo, khi)) continue;
+                for (unsigned spins = 0; (lds32(ga + 8 * s) & 63u) == kBusy;)  // its heads are being written
+                    if (++spins > kSpinLimit) return kGaveUp;
+                __threadfence_block();
+                bool same = true;
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            unsigned long long ct = s ? b.x : a.x, ch = s ? b.y : a.y;
-            if (ct == 0ull) {  // empty (or still being claimed): try to claim it
-                unsigned long long ot, oh;
-                cas128_shared(grp + 2 * s, ktail, head, ot, oh);
-                if (ot == 0ull && oh == 0ull) return (int)(2 * g + s);
-                ct = ot;
-                ch = oh;
+                for (int w = 0; w < W - 1; ++w) same = same && lds64(head_addr<W>(t, w, 2 * g + s)) == rec[w];
+                if (same) return (int)(2 * g + s);
             }
-            if (ct != ktail) continue;
-            if (ch != head) {
-                unsigned long long ot, oh;
-                cas128_shared(grp + 2 * s, 0ull, 0ull, ot, oh);  // the slot is claimed: no change, exact read
-                if (ot != ktail || oh != head) continue;
+            if (occ < GS) {
+                if (claim64(ga + 8 * occ, ktail | kBusy) != 0ull) continue;  // taken: the group is read again
+#pragma unroll
+                for (int w = 0; w < W - 1; ++w) sts64(head_addr<W>(t, w, 2 * g + occ), rec[w]);
+                __threadfence_block();
+                sts64(ga + 8 * occ, ktail);
+                return kClaimed;
             }
-            return (int)(2 * g + s);
         }
-        g = g + 1 == ngroups ? 0 : g + 1;
+        ++it;
+        g += (hsh >> 8 & 255u) | 1u;  // at least 256 groups: 64 steps never meet again
+        g -= g >= ngroups ? ngroups : 0u;
     }
-    return -1;
+    return kNoSlot;
 }
 
 template <int W>
-__device__ __forceinline__ void insert_record(const Table& t, const unsigned long long (&rec)[W], unsigned ngroups,
-                                              unsigned* s_flags) {
-    const unsigned long long tail = rec[W - 1];
-    const unsigned long long ktail = (tail & ~63ull) | kKeyMark;
-    // home group from every in-leaf bit of z (for short keys the top bits of the
-    // low word are partition bits, constant within a leaf): multiplicative hash
-    const unsigned long long zl = tail >> 6;
-    const unsigned hsh = (unsigned)((zl * 0x9E3779B97F4A7C15ull) >> 32);
-    unsigned g = (unsigned)(((unsigned long long)hsh * ngroups) >> 32);
-    int found = -1;
-    if (W == 2) found = find_slot2(t, ktail, rec[0], g, ngroups);
-    for (unsigned probe = 0; W != 2 && probe < kMaxGroupProbes && found < 0; ++probe) {
-        unsigned long long* grp = t.tail + 4 * g;
-        const ulonglong2 a = lds_v2_volatile(grp);
-        const ulonglong2 b = lds_v2_volatile(grp + 2);
-        unsigned long long cur[4] = {a.x, a.y, b.x, b.y};
-        for (int s = 0; s < 4 && found < 0; ++s) {
-            unsigned long long c = cur[s];
-            if (c == 0ull) {  // first empty slot of the group: try to claim it
-                const unsigned long long prev = atomicCAS(&grp[s], 0ull, W == 1 ? ktail : (ktail | kBusy));
-                if (prev == 0ull) {
-                    if (W > 1) {
-#pragma unroll
-                        for (int w = 0; w < W - 1; ++w) t.heads[(size_t)w * t.stride + 4 * g + s] = rec[w];
-                        __threadfence_block();
-                        atomicExch(&grp[s], ktail);
-                    }
-                    found = (int)(4 * g + s);
-                    break;
+__device__ __forceinline__ void count_record(const Table& t, const unsigned long long (&rec)[W], bool have,
+                                             unsigned ngroups, unsigned* s_flags) {
+    if constexpr (W == 1) {
+        // one loop with one exit: here the warp stays together (one-word rounds are
+        // short; leaving one by one cost 20.5 ms against 14.3 on 1.6 G windows, and
+        // staying together cost two-word keys 1.74 ms against 1.39 on 0.19 G)
+        const unsigned lo = (unsigned)rec[0], khi = (unsigned)(rec[0] >> 32), klo = lo + 1u;
+        const unsigned hsh = (lo & ~63u) * 0x9E3779B1u + khi * 0x85EBCA77u;
+        unsigned g = __umulhi(hsh, ngroups), it = 0, sl = 0;
+        bool pending = have, hit = false;
+        while (pending) {
+            const unsigned ga = t.tail + 16 * g;
+            const uint4 a = lds128(ga);
+            const bool e0 = same_tail(a.x, a.y, klo, khi), e1 = same_tail(a.z, a.w, klo, khi);
+            hit = e0 || e1;
+            const bool full = !hit && a.z != 0u;
+            pending = full;
+            sl = 2 * g + (e1 ? 1u : 0u);
+            if (!hit && a.z == 0u) {
+                const unsigned occ = a.x ? 1u : 0u;
+                const unsigned long long old = claim64(ga + 8 * occ, rec[0] + 1ull);
+                if (old != 0ull) {  // taken: by this key, or by another (the group is read again)
+                    sl = 2 * g + occ;
+                    hit = same_tail((unsigned)old, (unsigned)(old >> 32), klo, khi);
+                    pending = !hit;
                 }
-                c = prev;
             }
-            if ((c & ~kBusy) != ktail) continue;
-            if (W == 1) {
-                found = (int)(4 * g + s);
-                break;
-            }
-            unsigned spins = 0;
-            while (c & kBusy) {
-                if (++spins > kSpinLimit) {
-                    atomicOr(s_flags, kLeafTimeout);
-                    return;
+            if (full) {
+                g += (hsh >> 8 & 255u) | 1u;
+                g -= g >= ngroups ? ngroups : 0u;
+                if (++it == kMaxRounds) {
+                    pending = false;
+                    atomicOr(s_flags, kLeafFull);
                 }
-                c = *(volatile unsigned long long*)&grp[s];
             }
-            __threadfence_block();
-            bool same = true;
-#pragma unroll
-            for (int w = 0; w < W - 1; ++w)
-                same = same && (*(volatile unsigned long long*)&t.heads[(size_t)w * t.stride + 4 * g + s] == rec[w]);
-            if (same) found = (int)(4 * g + s);
         }
-        g = g + 1 == ngroups ? 0 : g + 1;
+        if (hit) {
+            const unsigned l = ext_left(lo), r = ext_right(lo);
+            bump(t, sl, l ? l - 1 : 4u);  // every counted window has exactly one left lane (the first: its code)
+            if (r) bump(t, sl, 4u + r);
+        }
+        __syncwarp();
+    } else {
+        int slot = kClaimed;
+        if (have) slot = find_slot<W>(t, rec, ngroups);
+        if (slot >= 0) {
+            const unsigned l = ext_left(rec[W - 1]), r = ext_right(rec[W - 1]);
+            bump(t, (unsigned)slot, l ? l - 1 : 4u);
+            if (r) bump(t, (unsigned)slot, 4u + r);
+        } else if (slot != kClaimed) {
+            atomicOr(s_flags, slot == kGaveUp ? kLeafTimeout : kLeafFull);
+        }
+        __syncwarp();
     }
-    if (found < 0) {
-        atomicOr(s_flags, kLeafFull);
-        return;
-    }
-    const unsigned l = ext_left(tail), r = ext_right(tail);
-    bump(t, (unsigned)found, l ? l - 1 : 4u);  // every window has exactly one left lane
-    if (r) bump(t, (unsigned)found, 4u + r);
 }
 
-// Clears slots [0, cap) of the table (all threads of the CTA).
+// Clears a warp's slice [s0, s0 + per) of the table (per a multiple of 32).
 template <int W>
-__device__ __forceinline__ void clear_slots(const Table& t, unsigned cap) {
-    for (unsigned s = threadIdx.x; s < cap; s += kLeafThreads) {
-        clear_key<W>(t, s);
+__device__ __forceinline__ void clear_slice(const Table& t, unsigned s0, unsigned per) {
+    const unsigned lane = threadIdx.x & 31;
+    // keys: tails, or (tail, head) pairs; head planes of empty slots are never read
+    const unsigned k = t.tail + (W == 2 ? 16 : 8) * s0, l = t.lanes + 4 * s0;
+    for (unsigned i = 16 * lane; i < (W == 2 ? 16 : 8) * per; i += 512) sts128_zero(k + i);
+    for (unsigned i = 16 * lane; i < 4 * per; i += 512) {
 #pragma unroll
-        for (unsigned p = 0; p < kLanePlanes; ++p) t.lanes[p * t.stride + s] = 0u;
+        for (unsigned p = 0; p < kLanePlanes; ++p) sts128_zero(l + 4 * p * t.stride + i);
     }
+}
+
+// Clears the whole table (all threads of the CTA; cap a multiple of 512).
+template <int W>
+__device__ __forceinline__ void clear_table(const Table& t, unsigned cap) {
+    clear_slice<W>(t, (threadIdx.x >> 5) * (cap / kLeafWarps), cap / kLeafWarps);
 }
 
 // Sweeps slots [0, cap): k-mers below min_count are dropped, survivors are
 // classified and written (one output reservation per warp), and every slot
-// is left clear.  Each warp takes a slice of cap / 16 slots.
+// is left clear.  Each warp takes a slice of cap / 16 slots: it lists its
+// survivors (four slots per lane and step, so that a slice takes two or three
+// steps), writes them with full warps, and clears the slice with 16-byte
+// stores.
 template <int W>
 __device__ __forceinline__ void sweep_table(const Job& j, const Table& t, const LeafInfo& li, unsigned cap,
-                                            unsigned long long& distinct) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned cap_max = t.stride;
+                                            unsigned& distinct) {
+    const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned plane = 4 * t.stride;
     const unsigned per = cap / kLeafWarps;  // a multiple of 32
     const unsigned s0 = wid * per;
-    unsigned* mylist = t.list + s0;
+    const unsigned more = j.min_count - 1;  // records besides the one that claimed the slot
+    const unsigned mylist = t.list + 4 * s0, before = (1u << lane) - 1u;
     unsigned count = 0;
-    for (unsigned s = s0 + lane; s < s0 + per; s += 32) {
-        const unsigned long long tl = slot_tail<W>(t, s);
-        const unsigned p0 = t.lanes[s], p1 = t.lanes[cap_max + s], p2 = t.lanes[2 * cap_max + s];
-        const unsigned c = (p0 & 0xFFFFu) + (p0 >> 16) + (p1 & 0xFFFFu) + (p1 >> 16) + (p2 & 0xFFFFu);
-        const bool ok = tl != 0ull && c >= j.min_count;
-        distinct += tl != 0ull ? 1 : 0;
-        const unsigned m = __ballot_sync(0xffffffffu, ok);
-        if (ok) {
-            mylist[count + __popc(m & ((1u << lane) - 1u))] = s;
-        } else {
-            clear_key<W>(t, s);
+    for (unsigned b = 0; b < per; b += 128) {
+        unsigned occ[4], p0[4], p1[4], p2[4];
+        // W = 2: keys are 16 bytes a slot, so neighbouring lanes take neighbouring slots
+        if constexpr (W == 2) {
 #pragma unroll
-            for (unsigned p = 0; p < kLanePlanes; ++p) t.lanes[p * cap_max + s] = 0u;
+            for (unsigned q = 0; q < 4; ++q) {
+                const unsigned o = b + 32 * q + lane, s = s0 + o;
+                occ[q] = p0[q] = p1[q] = p2[q] = 0u;
+                if (o < per) {
+                    occ[q] = lds32(t.tail + 16 * s);
+                    p0[q] = lds32(t.lanes + 4 * s);
+                    p1[q] = lds32(t.lanes + plane + 4 * s);
+                    p2[q] = lds32(t.lanes + 2 * plane + 4 * s);
+                }
+            }
+        } else {
+            const unsigned o = b + 4 * lane, s = s0 + o;
+            uint4 x = make_uint4(0u, 0u, 0u, 0u), y = x, a0 = x, a1 = x, a2 = x;
+            if (o < per) {
+                x = lds128(t.tail + 8 * s);
+                y = lds128(t.tail + 8 * s + 16);
+                a0 = lds128(t.lanes + 4 * s);
+                a1 = lds128(t.lanes + plane + 4 * s);
+                a2 = lds128(t.lanes + 2 * plane + 4 * s);
+            }
+            occ[0] = x.x; occ[1] = x.z; occ[2] = y.x; occ[3] = y.z;
+            p0[0] = a0.x; p0[1] = a0.y; p0[2] = a0.z; p0[3] = a0.w;
+            p1[0] = a1.x; p1[1] = a1.y; p1[2] = a1.z; p1[3] = a1.w;
+            p2[0] = a2.x; p2[1] = a2.y; p2[2] = a2.z; p2[3] = a2.w;
         }
-        count += __popc(m);
+#pragma unroll
+        for (unsigned q = 0; q < 4; ++q) {
+            // the five left lanes, two halves at a time (their sum is below 65536: no carry)
+            const unsigned h = p0[q] + p1[q] + (p2[q] & 0xFFFFu);
+            const bool ok = occ[q] != 0u && (h & 0xFFFFu) + (h >> 16) >= more;
+            distinct += occ[q] != 0u ? 1u : 0u;
+            const unsigned m = __ballot_sync(0xffffffffu, ok);
+            if (ok)
+                sts32(mylist + 4 * (count + __popc(m & before)), s0 + (W == 2 ? b + 32 * q + lane : b + 4 * lane + q));
+            count += __popc(m);
+        }
     }
     __syncwarp();
     unsigned long long wbase = 0;
     if (lane == 0 && count) wbase = atomicAdd(j.out_n, (unsigned long long)count);
     wbase = __shfl_sync(0xffffffffu, wbase, 0);
     for (unsigned i = lane; i < count; i += 32) {
-        const unsigned s = mylist[i];
+        const unsigned s = lds32(mylist + 4 * i);
         const unsigned long long pos = wbase + i;
         const unsigned long long tl = slot_tail<W>(t, s);
         unsigned pl[kLanePlanes];
 #pragma unroll
-        for (unsigned p = 0; p < kLanePlanes; ++p) pl[p] = t.lanes[p * cap_max + s];
+        for (unsigned p = 0; p < kLanePlanes; ++p) pl[p] = lds32(t.lanes + p * plane + 4 * s);
         unsigned long long key[W];
 #pragma unroll
-        for (int w = 0; w < W - 1; ++w) key[w] = slot_head<W>(t, w, s);
-        clear_key<W>(t, s);
-#pragma unroll
-        for (unsigned p = 0; p < kLanePlanes; ++p) t.lanes[p * cap_max + s] = 0u;
+        for (int w = 0; w < W - 1; ++w) key[w] = lds64(head_addr<W>(t, w, s));
         if (pos >= j.out_cap) {
             set_status(j, ST_OUT_OVERFLOW);
             continue;
         }
-        const unsigned nl[4] = {pl[0] & 0xFFFFu, pl[0] >> 16, pl[1] & 0xFFFFu, pl[1] >> 16};
-        const unsigned nr[4] = {pl[2] >> 16, pl[3] & 0xFFFFu, pl[3] >> 16, pl[4] & 0xFFFFu};
-        const unsigned c = nl[0] + nl[1] + nl[2] + nl[3] + (pl[2] & 0xFFFFu);
+        unsigned nl[4] = {pl[0] & 0xFFFFu, pl[0] >> 16, pl[1] & 0xFFFFu, pl[1] >> 16};
+        unsigned nr[4] = {pl[2] >> 16, pl[3] & 0xFFFFu, pl[3] >> 16, pl[4] & 0xFFFFu};
+        const unsigned c = 1u + nl[0] + nl[1] + nl[2] + nl[3] + (pl[2] & 0xFFFFu);
+        const unsigned code = ((unsigned)tl & 63u) - 1u, fl = ext_left(code), fr = ext_right(code);  // the first record
+#pragma unroll
+        for (unsigned b = 0; b < 4; ++b) {
+            nl[b] += fl == b + 1u ? 1u : 0u;
+            nr[b] += fr == b + 1u ? 1u : 0u;
+        }
         const unsigned long long z = record_z(j.g, j.pass, j.bucket0 + li.bucket, tl);
         key[W - 1] = z_to_tail<W>(z, key, j.g.bt);
 #pragma unroll
@@ -334,6 +440,8 @@ __device__ __forceinline__ void sweep_table(const Job& j, const Table& t, const 
         eo[1] = make_uint4(nr[0], nr[1], nr[2], nr[3]);
         reinterpret_cast<uchar2*>(j.out_cls)[pos] = make_uchar2(classify_side(nl, c, j), classify_side(nr, c, j));
     }
+    __syncwarp();
+    clear_slice<W>(t, s0, per);
 }
 
 // A leaf whose keys did not fit its table (and that has fewer than 65 536
@@ -346,8 +454,8 @@ __device__ __forceinline__ void sweep_table(const Job& j, const Table& t, const 
 // counted.
 template <int W>
 __device__ __forceinline__ unsigned count_in_ranges(const Job& j, const Table& t, const LeafInfo& li, unsigned leaf,
-                                                 unsigned* s_flags, unsigned long long* distinct) {
-    const unsigned long long n = li.n;
+                                                 unsigned* s_flags, unsigned* distinct) {
+    const unsigned n = (unsigned)li.n;  // below 65 536
     const unsigned zb = j.g.zl_bits();
     const unsigned free_bits = zb > j.g.p2 ? zb - j.g.p2 : 0u;  // z bits below the leaf's
     const unsigned max_rb = free_bits < kMaxSubBits ? free_bits : kMaxSubBits;
@@ -358,19 +466,20 @@ __device__ __forceinline__ unsigned count_in_ranges(const Job& j, const Table& t
     for (;;) {
         const unsigned shift = free_bits - rb, rmask = (1u << rb) - 1u;
         unsigned rwin = 0;
-        for (unsigned long long i = threadIdx.x; i < n; i += kLeafThreads) {
+        for (unsigned i0 = 0; i0 < n; i0 += kLeafThreads) {
+            const unsigned i = i0 + threadIdx.x;
             unsigned long long rec[W];
 #pragma unroll
-            for (int w = 0; w < W; ++w) rec[w] = src[i * W + w];
-            if (((unsigned)((rec[W - 1] >> 6) >> shift) & rmask) != rs) continue;
-            ++rwin;
-            if (!*(volatile unsigned*)s_flags) insert_record<W>(t, rec, groups_of<W>(cap), s_flags);
+            for (int w = 0; w < W; ++w) rec[w] = i < n ? src[(size_t)i * W + w] : 0ull;
+            const bool in = i < n && ((unsigned)((rec[W - 1] >> 6) >> shift) & rmask) == rs;
+            rwin += in ? 1u : 0u;
+            count_record<W>(t, rec, in && !*(volatile unsigned*)s_flags, groups_of<W>(cap), s_flags);
         }
         __syncthreads();
         const unsigned flags = *(volatile unsigned*)s_flags;
         if (flags == kLeafFull && rb < max_rb) {  // split the range in two
             if (threadIdx.x == 0 && rb == 0) atomicAdd(j.stats + 3, 1ull);
-            clear_slots<W>(t, cap);
+            clear_table<W>(t, cap);
             __syncthreads();
             if (threadIdx.x == 0) *s_flags = 0;
             __syncthreads();
@@ -388,7 +497,7 @@ __device__ __forceinline__ unsigned count_in_ranges(const Job& j, const Table& t
                     else set_status(j, ST_FALLBACK_FULL);
                 }
             }
-            clear_slots<W>(t, cap);
+            clear_table<W>(t, cap);
         } else {
             windows += rwin;
             sweep_table<W>(j, t, li, cap, *distinct);
@@ -419,22 +528,23 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_split_kernel(const Job* 
     const int lane = threadIdx.x & 31;
     Table t;
     t.stride = cap_max;
-    t.tail = reinterpret_cast<unsigned long long*>(smem);
-    t.heads = t.tail + cap_max;
-    t.lanes = reinterpret_cast<unsigned*>(t.heads + (size_t)(W - 1) * cap_max);
-    t.list = t.lanes + (size_t)kLanePlanes * cap_max;
+    t.tail = (unsigned)__cvta_generic_to_shared(smem);
+    t.heads = t.tail + 8 * cap_max;
+    t.lanes = t.heads + 8 * (W - 1) * cap_max;
+    t.list = t.lanes + 4 * kLanePlanes * cap_max;
     bool init = false;
     for (unsigned ji = 0; ji < n_jobs; ++ji) {
         const Job& j = jobs[ji];
         const unsigned n_split = *(volatile unsigned*)j.split_n;
         if (blockIdx.x >= n_split) continue;
         if (!init) {
-            clear_slots<W>(t, cap_max);
+            clear_table<W>(t, cap_max);
             if (threadIdx.x == 0) s_flags = 0;
             __syncthreads();
             init = true;
         }
-        unsigned long long windows = 0, distinct = 0;
+        unsigned long long windows = 0;
+        unsigned distinct = 0;
         for (unsigned e = blockIdx.x; e < n_split; e += gridDim.x) {
             const unsigned leaf = j.split_list[e];
             const LeafInfo li = leaf_info(j, leaf);
@@ -459,24 +569,28 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_kernel(const Job* __rest
     constexpr int U = LeafShape<W>::U, B = LeafShape<W>::B;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned s_flags;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ Job s_job;        // the current analysis: its fields are read in every phase of every leaf
+    __shared__ LeafInfo s_next;  // the next leaf, looked up by one thread while this one is counted
+    const int lane = threadIdx.x & 31;
     const unsigned long long total = leaf_off[n_jobs];
+    static_assert(sizeof(Job) % 4 == 0, "copied word by word");
+    auto take_job = [&](unsigned ji) {
+        for (unsigned i = threadIdx.x; i < sizeof(Job) / 4; i += kLeafThreads)
+            reinterpret_cast<unsigned*>(&s_job)[i] = reinterpret_cast<const unsigned*>(jobs + ji)[i];
+    };
 
     Table t;
     t.stride = cap_max;
-    t.tail = reinterpret_cast<unsigned long long*>(smem);
-    t.heads = t.tail + cap_max;
-    t.lanes = reinterpret_cast<unsigned*>(t.heads + (size_t)(W - 1) * cap_max);
-    t.list = t.lanes + (size_t)kLanePlanes * cap_max;
-    for (unsigned s = threadIdx.x; s < cap_max; s += kLeafThreads) {
-        clear_key<W>(t, s);
-#pragma unroll
-        for (unsigned p = 0; p < kLanePlanes; ++p) t.lanes[p * cap_max + s] = 0u;
-    }
+    t.tail = (unsigned)__cvta_generic_to_shared(smem);
+    t.heads = t.tail + 8 * cap_max;
+    t.lanes = t.heads + 8 * (W - 1) * cap_max;
+    t.list = t.lanes + 4 * kLanePlanes * cap_max;
+    clear_table<W>(t, cap_max);
     if (threadIdx.x == 0) s_flags = 0;
 
     // statistics of the current analysis, added when the analysis changes
-    unsigned long long windows = 0, distinct = 0;
+    unsigned long long windows = 0;
+    unsigned distinct = 0;  // of this thread's slots: far below 2^32
     unsigned stat_job = 0;
     auto flush_stats = [&](unsigned ji) {
         unsigned long long d = distinct;
@@ -484,7 +598,8 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_kernel(const Job* __rest
         for (int o = 16; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
         if (lane == 0 && d) atomicAdd(jobs[ji].stats + 1, d);
         if (threadIdx.x == 0 && windows) atomicAdd(jobs[ji].stats + 0, windows);
-        windows = distinct = 0;
+        windows = 0;
+        distinct = 0;
     };
 
     unsigned long long g = blockIdx.x;
@@ -499,14 +614,18 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_kernel(const Job* __rest
         li = leaf_info(jobs[ji], leaf);
         load_batch<W>(li, 0, batch);
         stat_job = ji;
+        take_job(ji);
     }
     __syncthreads();
 
+    const Job& j = s_job;
     while (g < total) {
-        const Job& j = jobs[ji];
         if (ji != stat_job) {
             flush_stats(stat_job);
             stat_job = ji;
+            __syncthreads();  // every thread is done with the previous analysis
+            take_job(ji);
+            __syncthreads();
         }
         const unsigned long long ng = g + gridDim.x;
         unsigned nji = ji, nleaf = 0;
@@ -530,29 +649,29 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_kernel(const Job* __rest
             continue;
         }
         // ---------------------------------------------------------- count
-        const unsigned long long n = li.n;
-        const unsigned long long want = ((n * j.table_ratio_num) >> 16) + 512;
-        const unsigned cap = (unsigned)(want < cap_max ? ((want + 511) & ~511ull) : cap_max);
+        const unsigned n = (unsigned)li.n;  // below 65 536, as is the ratio (at most 65 536)
+        const unsigned want = (unsigned)(((unsigned long long)n * j.table_ratio_num) >> 16) + 512u;
+        const unsigned cap = want < cap_max ? ((want + 511u) & ~511u) : cap_max;
         const unsigned ngroups = groups_of<W>(cap);
-        for (unsigned long long first = 0; first < n; first += B) {
+        if (threadIdx.x == kLeafThreads - 1) {
+            LeafInfo x;
+            x.ok = false;
+            if (ng < total) x = leaf_info(jobs[nji], nleaf);
+            s_next = x;
+        }
+        for (unsigned first = 0; first < n; first += B) {
             if (first) load_batch<W>(li, first, batch);
+            if (*(volatile unsigned*)&s_flags) break;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const unsigned long long i = first + (unsigned long long)u * kLeafThreads + threadIdx.x;
-                if (i < n && !*(volatile unsigned*)&s_flags) insert_record<W>(t, batch[u], ngroups, &s_flags);
+                count_record<W>(t, batch[u], first + u * kLeafThreads + threadIdx.x < n, ngroups, &s_flags);
             }
         }
         __syncthreads();
         const unsigned flags = s_flags;
         // the next leaf's first batch loads while this one is swept
-        LeafInfo nli;
-        nli.ok = false;
-        if (ng < total) {
-            nli = leaf_info(jobs[nji], nleaf);
-            load_batch<W>(nli, 0, batch);
-        }
-        const unsigned per = cap / kLeafWarps;  // a multiple of 32
-        const unsigned s0 = wid * per;
+        const LeafInfo nli = s_next;
+        load_batch<W>(nli, 0, batch);
         if (flags) {
             if (threadIdx.x == 0) {
                 if (flags & kLeafTimeout) {
@@ -568,11 +687,7 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_kernel(const Job* __rest
                     }
                 }
             }
-            for (unsigned s = s0 + lane; s < s0 + per; s += 32) {  // leave the table clean
-                clear_key<W>(t, s);
-#pragma unroll
-                for (unsigned p = 0; p < kLanePlanes; ++p) t.lanes[p * cap_max + s] = 0u;
-            }
+            clear_table<W>(t, cap);  // leave the table clean
         } else {
             if (threadIdx.x == 0) windows += n;
             sweep_table<W>(j, t, li, cap, distinct);  // filter, classify, compact (per warp)
