@@ -825,7 +825,8 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
             j.gate = h->gate2.as<unsigned long long>();
             j.gate_bits = h->gate_bits;
         }
-        // one scatter job per submitted readset, one CTA per 256 reads
+        // one scatter job per submitted readset, one CTA per tile of reads
+        const unsigned tile_reads = scatter_tile_reads(W);
         std::vector<Job> sjobs;
         std::vector<unsigned long long> tile_off(1, 0);
         for (const kmer_readset* rs : h->submitted) {
@@ -833,7 +834,7 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
             Job js = j;
             set_readset(js, rs);
             sjobs.push_back(js);
-            tile_off.push_back(tile_off.back() + (rs->n_reads + 255) / 256);
+            tile_off.push_back(tile_off.back() + (rs->n_reads + tile_reads - 1) / tile_reads);
         }
         TRY(upload(h, h->d_sjobs, sjobs));
         TRY(upload(h, h->d_tile_off, tile_off));

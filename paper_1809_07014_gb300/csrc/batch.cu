@@ -210,9 +210,10 @@ int capture_wave(kmer_batch* b, Wave& w) {
     std::vector<unsigned long long> host_maps;
     for (auto& c : w.classes) {
         std::vector<unsigned long long> tile_off(1, 0), leaf_off(1, 0);
+        const unsigned tile_reads = scatter_tile_reads(c.W);
         for (unsigned i = 0; i < c.count; ++i) {
             const BJob& j = b->jobs[w.ids[c.first + i]];
-            tile_off.push_back(tile_off.back() + (j.rs->n_reads + 255) / 256);
+            tile_off.push_back(tile_off.back() + (j.rs->n_reads + tile_reads - 1) / tile_reads);
             leaf_off.push_back(leaf_off.back() + (1ull << (j.g.p1 + j.g.p2)));
         }
         c.tiles = tile_off.back();

@@ -69,18 +69,19 @@ __host__ __device__ inline unsigned long long low_mask(unsigned b) {
 }
 
 // Hash of the head words (words 0..W-2) that is xored into the last word
-// before the multiply, so that z depends on the whole key.
+// before the multiply, so that z depends on the whole key: a multilinear hash
+// of their 32-bit halves (two multiply-adds a word), its high half folded
+// into the low one.
 template <int W>
 __host__ __device__ inline unsigned long long head_hash(const unsigned long long (&w)[W]) {
+    constexpr unsigned c[6] = {0x9E3779B1u, 0x85EBCA77u, 0xC2B2AE3Du, 0x27D4EB2Fu, 0x165667B1u, 0xD3A2646Du};
     unsigned long long h = 0x9E3779B97F4A7C15ull;
 #pragma unroll
     for (int i = 0; i < W - 1; ++i) {
-        h ^= w[i];
-        h ^= h >> 31;
-        h *= 0x94D049BB133111EBull;
-        h ^= h >> 29;
+        h += (w[i] & 0xFFFFFFFFull) * c[2 * i];
+        h += (w[i] >> 32) * c[2 * i + 1];
     }
-    return W > 1 ? h : 0ull;
+    return W > 1 ? h ^ (h >> 32) : 0ull;
 }
 
 // Geometry of one analysis: k-mer words, mixing width and partition bits.

@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(256) gate_kernel(const Job j, unsigned long lo
     if (r < j.n_reads) {
         Roll<W, HI> roll;
         roll.init(j, r);
-        for (unsigned long long t = 0; t <= roll.L; ++t) {
+        for (unsigned t = j.g.k; t <= roll.L; ++t) {
             unsigned long long key[W];
             unsigned lc, rc;
             if (!roll.step(t, key, lc, rc)) continue;

@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) direct_insert_kernel(const Job j, HEntry<
     if (r < j.n_reads) {
         Roll<W> roll;
         roll.init(j, r);
-        for (unsigned long long step = 0; step <= roll.L; ++step) {
+        for (unsigned step = j.g.k; step <= roll.L; ++step) {
             unsigned long long key[W];
             unsigned lc, rc;
             if (roll.step(step, key, lc, rc)) {

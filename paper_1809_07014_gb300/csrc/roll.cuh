@@ -10,127 +10,109 @@
 
 namespace kmer {
 
+// A window's words a < b, word 0 most significant: one borrow chain, no branch.
+template <int W>
+__device__ __forceinline__ bool words_less(const unsigned long long (&a)[W], const unsigned long long (&b)[W]) {
+    if constexpr (W == 1) {
+        return a[0] < b[0];
+    } else {
+        unsigned r;
+        unsigned long long t;
+        if constexpr (W == 2)
+            asm("sub.cc.u64 %1, %2, %4;\n\tsubc.cc.u64 %1, %3, %5;\n\tsubc.u32 %0, 0, 0;"
+                : "=r"(r), "=&l"(t) : "l"(a[1]), "l"(a[0]), "l"(b[1]), "l"(b[0]));
+        else if constexpr (W == 3)
+            asm("sub.cc.u64 %1, %2, %5;\n\tsubc.cc.u64 %1, %3, %6;\n\tsubc.cc.u64 %1, %4, %7;\n\tsubc.u32 %0, 0, 0;"
+                : "=r"(r), "=&l"(t) : "l"(a[2]), "l"(a[1]), "l"(a[0]), "l"(b[2]), "l"(b[1]), "l"(b[0]));
+        else
+            asm("sub.cc.u64 %1, %2, %6;\n\tsubc.cc.u64 %1, %3, %7;\n\tsubc.cc.u64 %1, %4, %8;\n\t"
+                "subc.cc.u64 %1, %5, %9;\n\tsubc.u32 %0, 0, 0;"
+                : "=r"(r), "=&l"(t)
+                : "l"(a[3]), "l"(a[2]), "l"(a[1]), "l"(a[0]), "l"(b[3]), "l"(b[2]), "l"(b[1]), "l"(b[0]));
+        return r != 0u;
+    }
+}
+
+// The 32 bases of a word reversed and complemented.
+__device__ __forceinline__ unsigned long long revcomp_word(unsigned long long x) {
+    const unsigned long long m = __brevll(~x);
+    return ((m >> 1) & 0x5555555555555555ull) | ((m & 0x5555555555555555ull) << 1);
+}
+
+// One read's windows in order.  init() stands at the first window: its words
+// come from the packed blocks by shifts, its reverse complement by bit
+// reversal and the last N before it from the N masks, so the k bases of the
+// first window cost no steps (two thirds of a 150-base read's steps at
+// k = 99, a fifth at k = 31).
+//
 // HI (one word, k >= 17): the window's first base sits in the high 32 bits
 // of the word, so the base leaving the window and the complement entering the
 // reverse strand touch that half only.
 template <int W, bool HI = false>
 struct Roll {
     unsigned long long fwd[W], rc[W];
-    unsigned long long gh0, gh1;  // good bits of the last 128 bases, bit m = base t-1-m
-    long long last_n;             // last position holding an N (or -1)
-    unsigned long long cur;       // bases of the current block, next base in the top 2 bits
-    unsigned curn, curg;          // N / good bits of the current block, next base in bit 0
-    uint4 nxt;                    // the block after the current one, loaded one block ahead
-    unsigned out;                 // base that left the window at the last step
+    unsigned long long cur;        // bases of the current block, next base in the top 2 bits
+    unsigned curn, curg;           // N / good bits of the current block, next base in bit 0
+    unsigned lg, lgn;              // good bits of the bases that left the window, next in bit 0; the block after
+    uint4 nxt;                     // the block after the current one, loaded one block ahead
+    unsigned out;                  // base that left the window at the last step
+    unsigned L, k, sh;             // sh: shift of the window's first base within its 32-bit half
+    unsigned first_ok;             // first step whose window holds no N: last N position + k + 1
     const PackedBlock* blk;
-    unsigned long long L;
-    unsigned k, hb;
-    unsigned long long topmask;
+    unsigned long long mask;       // bits of word 0
 
+    // Stands before step k (reads shorter than k have no steps).
     __device__ void init(const Job& j, unsigned long long r) {
         const unsigned long long a = j.offsets[r];
-        L = j.offsets[r + 1] - a;
+        L = (unsigned)(j.offsets[r + 1] - a);  // reads are shorter than 2^31 bases
         blk = j.blocks + j.blk_off[r];
         k = j.g.k;
-        hb = j.g.hb;
-        topmask = low_mask(hb);
-#pragma unroll
-        for (int i = 0; i < W; ++i) { fwd[i] = 0; rc[i] = 0; }
-        gh0 = gh1 = 0;
-        last_n = -1;
-        out = 0;
+        const unsigned hb = j.g.hb;
+        mask = low_mask(hb);
+        sh = hb - 2;
+        first_ok = k;
+        out = lg = lgn = 0;
         cur = 0;
         curn = curg = 0;
-        nxt = L ? __ldg(reinterpret_cast<const uint4*>(blk)) : make_uint4(0, 0, 0, 0);
+        nxt = make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int i = 0; i < W; ++i) fwd[i] = rc[i] = 0;
+        if (L < k) return;
+        unsigned long long B[W];
+        unsigned last_n = 0;  // last N of the first k bases, plus one
+#pragma unroll
+        for (int i = 0; i < W; ++i) {  // k > 32 (W - 1): the first W blocks hold the first window
+            const uint4 x = __ldg(reinterpret_cast<const uint4*>(blk + i));
+            B[i] = (unsigned long long)x.y << 32 | x.x;
+            unsigned nm = x.z;
+            if (i == W - 1) {
+                const unsigned o = k - 32 * (W - 1);  // 1..31 bases of this block (k odd)
+                nm &= (1u << o) - 1u;
+                cur = B[i] << (2 * o);
+                curn = x.z >> o;
+                curg = x.w >> o;
+            }
+            if (nm) last_n = 32 * i + 32 - __clz(nm);
+            if (i == 0) lgn = x.w;
+        }
+        if (last_n) first_ok = last_n + k;
+        if (32u * W < L) nxt = __ldg(reinterpret_cast<const uint4*>(blk + W));
+        fwd[0] = B[0] >> (64 - hb);
+#pragma unroll
+        for (int i = 1; i < W; ++i) fwd[i] = (B[i - 1] << hb) | (B[i] >> (64 - hb));
+        unsigned long long R[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) R[i] = revcomp_word(fwd[W - 1 - i]);
+        rc[0] = R[0] >> (64 - hb);
+#pragma unroll
+        for (int i = 1; i < W; ++i) rc[i] = (R[i - 1] << hb) | (R[i] >> (64 - hb));
     }
 
-    // Step t (0 <= t <= L).  First the window [t-k, t) is reported if t >= k
-    // and it holds no N; then base t (if t < L) is shifted in.  Returns true
-    // and fills key / lcode / rcode (0 = none, 1..4 = A..T) for a window.
-    __device__ __forceinline__ bool step(unsigned long long t, unsigned long long (&key)[W], unsigned& lcode,
-                                         unsigned& rcode) {
-        unsigned b = 0, good = 0, isn = 0;
-        if (t < L) {
-            if ((t & 31) == 0) {
-                cur = ((unsigned long long)nxt.y << 32) | nxt.x;
-                curn = nxt.z;
-                curg = nxt.w;
-                if (t + 32 < L) nxt = __ldg(reinterpret_cast<const uint4*>(blk + (t >> 5) + 1));
-            }
-            b = (unsigned)(cur >> 62);
-            cur <<= 2;
-            isn = curn & 1u;
-            curn >>= 1;
-            good = curg & 1u;
-            curg >>= 1;
-        }
-        bool emit = false;
-        if (t >= k && last_n < (long long)(t - k)) {
-            emit = true;
-            // the history holds zeros before the read's first base, so the
-            // first window finds no left extension, and `good` is 0 past the end
-            const unsigned lgood = k < 64 ? (unsigned)(gh0 >> k) & 1u : (unsigned)(gh1 >> (k - 64)) & 1u;
-            unsigned lc = lgood ? out + 1 : 0;
-            unsigned rcd = good ? b + 1 : 0;
-            // canonical: the lexicographically smaller of forward and reverse complement
-            bool flip = false;
-#pragma unroll
-            for (int w = 0; w < W; ++w) {
-                if (fwd[w] != rc[w]) { flip = rc[w] < fwd[w]; break; }
-            }
-#pragma unroll
-            for (int w = 0; w < W; ++w) key[w] = flip ? rc[w] : fwd[w];
-            if (flip) {  // the key reads the other strand: swap sides, complement bases
-                const unsigned nl = rcd ? 5 - rcd : 0, nr = lc ? 5 - lc : 0;
-                lc = nl;
-                rcd = nr;
-            }
-            lcode = lc;
-            rcode = rcd;
-        }
-        if (t < L) {
-            out = (unsigned)(fwd[0] >> (hb - 2)) & 3u;
-#pragma unroll
-            for (int w = 0; w < W - 1; ++w) fwd[w] = (fwd[w] << 2) | (fwd[w + 1] >> 62);
-            fwd[W - 1] = (fwd[W - 1] << 2) | b;
-            fwd[0] &= topmask;
-#pragma unroll
-            for (int w = W - 1; w > 0; --w) rc[w] = (rc[w] >> 2) | (rc[w - 1] << 62);
-            rc[0] = (rc[0] >> 2) | ((unsigned long long)(3u - b) << (hb - 2));
-            gh1 = (gh1 << 1) | (gh0 >> 63);
-            gh0 = (gh0 << 1) | good;
-            if (isn) last_n = (long long)t;
-        }
-        return emit;
-    }
-};
-
-// k <= 31: the whole k-mer fits one word; positions and the quality history
-// fit 32 bits (reads are shorter than 2^31 bases).
-template <bool HI>
-struct Roll<1, HI> {
-    unsigned long long fwd, rc, mask, cur;
-    unsigned curn, curg, gh, out, L, k, sh;
-    int first_ok;  // first step whose window holds no N: last N position + k + 1
-    uint4 nxt;
-    const PackedBlock* blk;
-
-    __device__ void init(const Job& j, unsigned long long r) {
-        const unsigned long long a = j.offsets[r];
-        L = (unsigned)(j.offsets[r + 1] - a);
-        blk = j.blocks + j.blk_off[r];
-        k = j.g.k;
-        sh = 2 * k - 2;
-        mask = low_mask(2 * k);
-        fwd = rc = cur = 0;
-        curn = curg = gh = out = 0;
-        first_ok = (int)k;
-        nxt = L ? __ldg(reinterpret_cast<const uint4*>(blk)) : make_uint4(0, 0, 0, 0);
-    }
-
-    __device__ __forceinline__ bool step(unsigned long long t64, unsigned long long (&key)[1], unsigned& lcode,
-                                         unsigned& rcode) {
-        const unsigned t = (unsigned)t64;
+    // Step t = k, k + 1, ..., L, in order.  First the window [t-k, t) is
+    // reported if it holds no N; then base t (if t < L) is shifted in.
+    // Returns true and fills key / lcode / rcode (0 = none, 1..4 = A..T) for a
+    // window.
+    __device__ __forceinline__ bool step(unsigned t, unsigned long long (&key)[W], unsigned& lcode, unsigned& rcode) {
         const bool in = t < L;
         unsigned b = 0, good = 0, isn = 0;
         if (in) {
@@ -147,14 +129,24 @@ struct Roll<1, HI> {
             good = curg & 1u;
             curg >>= 1;
         }
-        bool emit = false;
-        if ((int)t >= first_ok) {
-            emit = true;
-            // gh is zero before the first base and `good` is 0 past the end
-            unsigned lc = ((gh >> k) & 1u) ? out + 1 : 0;
+        // the base before the window, t - k - 1: none at the first step (lg starts at 0);
+        // base q = t - k leaves the window now and is next in lg
+        const unsigned lgood = lg & 1u;
+        const unsigned q = t - k;
+        if ((q & 31) == 0) {
+            lg = lgn;
+            if (q + 32 < L) lgn = __ldg(&blk[(q >> 5) + 1].hqmask);
+        } else {
+            lg >>= 1;
+        }
+        const bool emit = t >= first_ok;
+        if (emit) {
+            unsigned lc = lgood ? out + 1 : 0;
             unsigned rcd = good ? b + 1 : 0;
-            const bool flip = rc < fwd;
-            key[0] = flip ? rc : fwd;
+            // canonical: the lexicographically smaller of forward and reverse complement
+            const bool flip = words_less<W>(rc, fwd);
+#pragma unroll
+            for (int w = 0; w < W; ++w) key[w] = flip ? rc[w] : fwd[w];
             if (flip) {  // the key reads the other strand: swap sides, complement bases
                 const unsigned nl = rcd ? 5 - rcd : 0, nr = lc ? 5 - lc : 0;
                 lc = nl;
@@ -165,15 +157,18 @@ struct Roll<1, HI> {
         }
         if (in) {
             if (HI) {
-                out = ((unsigned)(fwd >> 32) >> (sh - 32)) & 3u;
-                rc = (rc >> 2) | ((unsigned long long)((3u - b) << (sh - 32)) << 32);
+                out = ((unsigned)(fwd[0] >> 32) >> (sh - 32)) & 3u;
             } else {
-                out = (unsigned)(fwd >> sh) & 3u;
-                rc = (rc >> 2) | ((unsigned long long)(3u - b) << sh);
+                out = (unsigned)(fwd[0] >> sh) & 3u;
             }
-            fwd = ((fwd << 2) | b) & mask;
-            gh = (gh << 1) | good;
-            if (isn) first_ok = (int)(t + k + 1);
+#pragma unroll
+            for (int w = 0; w < W - 1; ++w) fwd[w] = (fwd[w] << 2) | (fwd[w + 1] >> 62);
+            fwd[W - 1] = (fwd[W - 1] << 2) | b;
+            fwd[0] &= mask;
+#pragma unroll
+            for (int w = W - 1; w > 0; --w) rc[w] = (rc[w] >> 2) | (rc[w - 1] << 62);
+            rc[0] = (rc[0] >> 2) | (HI ? (unsigned long long)((3u - b) << (sh - 32)) << 32 : (unsigned long long)(3u - b) << sh);
+            if (isn) first_ok = t + k + 1;
         }
         return emit;
     }

@@ -3,6 +3,13 @@
 // top bits of the mixed key.  This is the all-to-all k-mer exchange of the
 // paper's k-mer analysis (Sec. II-B), done as a device-wide partition in HBM:
 // a bucket plays the role of the owning processor.
+//
+// Bound by issue slots (integer work of the windows, then the staging of the
+// records), not by DRAM.  A thread starts at its read's first window (Roll)
+// and a round's steps are unrolled, so the records' meta words stay in
+// registers; three CTAs per SM.  2-Gbase reads at k = 31: 11.45 -> 9.08 ms
+// (176 G windows/s); 300 Mbases at k = 99: 3.05 -> 1.21 ms; 100 Mbases at
+// k = 77: 1.43 -> 0.92 ms.  512 threads and 8 positions a round: 10.4 ms.
 #include "kernels.h"
 #include "roll.cuh"
 #include "stage.cuh"
@@ -11,9 +18,10 @@ namespace kmer {
 
 template <int W>
 struct ScatterShape {
-    // read positions per round: 4096 records (W = 1) or about 48 KB of records staged
-    static constexpr unsigned R = W == 1 ? 16 : (W == 2 ? 12 : (W == 3 ? 8 : 6));
-    static constexpr unsigned S = R * kStageThreads;                 // staged records per round
+    // threads of a CTA (three CTAs per SM), read positions per round, staged records per round
+    static constexpr unsigned NT = 256, CTAS = 3;
+    static constexpr unsigned R = W == 1 ? 16 : (W == 2 ? 10 : (W == 3 ? 8 : 7));
+    static constexpr unsigned S = R * NT;
 };
 
 struct L1Dest {
@@ -25,57 +33,61 @@ struct L1Dest {
     __device__ unsigned long long cap(unsigned d) const { return __ldg(capp + d); }
 };
 
-// One CTA: 256 consecutive reads of job j (a read tile).
-// MAXPER: destinations handled by one thread in a flush (fan-out / 256).
+// One CTA: NT consecutive reads of job j (a read tile).
+// MAXPER: destinations handled by one thread in a flush (fan-out / NT).
 template <int W, unsigned MAXPER, bool HI, bool GATE>
 __device__ __forceinline__ void scatter_tile(const Job& j, const unsigned long long r0, const unsigned long long r1,
                                              unsigned char* smem) {
-    constexpr unsigned R = ScatterShape<W>::R, S = ScatterShape<W>::S;
+    constexpr unsigned R = ScatterShape<W>::R, S = ScatterShape<W>::S, NT = ScatterShape<W>::NT;
     __shared__ unsigned s_maxlen;
     const unsigned P = 1u << j.g.p1;
     StageBufs b = carve_stage(smem, W, S, P);
     if (threadIdx.x == 0) s_maxlen = 0;
-    for (unsigned d = threadIdx.x; d < P; d += kStageThreads) b.hist[d] = 0;
+    for (unsigned d = threadIdx.x; d < P; d += NT) b.hist[d] = 0;
     __syncthreads();
 
     const unsigned long long r = r0 + threadIdx.x;
     Roll<W, HI> roll;
-    unsigned L = 0;  // reads are shorter than 2^31 bases
-    const bool have = r < r1;
-    if (have) {
-        roll.init(j, r);
-        L = (unsigned)roll.L;
-        atomicMax(&s_maxlen, (unsigned)L);
-    }
-    __syncthreads();
-    const unsigned rounds = (s_maxlen + R) / R;  // steps 0 .. maxlen
-    L1Dest dest{j.l1_fill, j.l1_start, j.l1_cap};
+    roll.L = 0;
     const Geometry g = j.g;
+    if (r < r1) {
+        roll.init(j, r);
+        atomicMax(&s_maxlen, roll.L);
+    }
+    const bool have = r < r1 && roll.L >= g.k;
+    __syncthreads();
+    const unsigned maxlen = s_maxlen;
+    L1Dest dest{j.l1_fill, j.l1_start, j.l1_cap};
     const unsigned pass = j.pass;
     const unsigned long long* gate = j.gate;  // Bloom gate (GATE): emit only keys in F2
     const unsigned gate_bits = j.gate_bits;
     unsigned emitted = 0;
-    for (unsigned round = 0; round < rounds; ++round) {
-#pragma unroll 2
+    for (unsigned t0 = g.k; t0 <= maxlen; t0 += R) {  // steps k .. maxlen
+        unsigned m[R];
+#pragma unroll
         for (unsigned s = 0; s < R; ++s) {
-            const unsigned t = round * R + s;
-            const unsigned e = s * kStageThreads + threadIdx.x;
-            unsigned m = 0xFFFFFFFFu;
-            if (have && t <= L) {
+            const unsigned t = t0 + s;
+            const unsigned e = s * NT + threadIdx.x;
+            m[s] = 0xFFFFFFFFu;
+            if (have && t <= roll.L) {
                 unsigned long long key[W], rec[W];
                 unsigned lc = 0, rc = 0, bucket = 0;
                 if (roll.step(t, key, lc, rc) && (!GATE || gate_has<W>(gate, gate_bits, key)) &&
                     make_record<W>(g, pass, key, lc, rc, rec, bucket)) {
-                    const unsigned rank = atomicAdd(&b.hist[bucket], 1u);
+                    m[s] = (bucket << 16) | atomicAdd(&b.hist[bucket], 1u);
+                    if constexpr (W == 2 || W == 4) {
 #pragma unroll
-                    for (int w = 0; w < W; ++w) b.stage[(size_t)e * W + w] = rec[w];
-                    m = (bucket << 16) | rank;
+                        for (int w = 0; w < W; w += 2)
+                            *reinterpret_cast<ulonglong2*>(b.stage + (size_t)e * W + w) = make_ulonglong2(rec[w], rec[w + 1]);
+                    } else {
+#pragma unroll
+                        for (int w = 0; w < W; ++w) b.stage[(size_t)e * W + w] = rec[w];
+                    }
                     ++emitted;
                 }
             }
-            b.meta[e] = m;
         }
-        flush_stage<W, MAXPER>(b, S, P, dest, j.l1_rec, j.status, ST_L1_OVERFLOW);
+        flush_stage_regs<W, MAXPER, L1Dest, NT, R>(b, S, P, dest, j.l1_rec, j.status, ST_L1_OVERFLOW, m);
     }
     // windows emitted into this pass (checked against the windows the leaves count)
 #pragma unroll
@@ -85,15 +97,25 @@ __device__ __forceinline__ void scatter_tile(const Job& j, const unsigned long l
 
 // One CTA per read tile over all jobs (all of key width W).
 template <int W, unsigned MAXPER, bool HI, bool GATE>
-__global__ void __launch_bounds__(kStageThreads, W == 1 ? 3 : 2)
+__global__ void __launch_bounds__(ScatterShape<W>::NT, ScatterShape<W>::CTAS)
 scatter_kernel(const Job* __restrict__ jobs, const unsigned long long* __restrict__ tile_off, const unsigned n_jobs) {
+    constexpr unsigned NT = ScatterShape<W>::NT;
     extern __shared__ __align__(16) unsigned char smem[];
     const unsigned long long t = blockIdx.x;
     const unsigned ji = job_of(tile_off, n_jobs, t);
     const Job& j = jobs[ji];
-    const unsigned long long r0 = (t - tile_off[ji]) * kStageThreads;
-    const unsigned long long r1 = r0 + kStageThreads < j.n_reads ? r0 + kStageThreads : j.n_reads;
+    const unsigned long long r0 = (t - tile_off[ji]) * NT;
+    const unsigned long long r1 = r0 + NT < j.n_reads ? r0 + NT : j.n_reads;
     scatter_tile<W, MAXPER, HI, GATE>(j, r0, r1, smem);
+}
+
+unsigned scatter_tile_reads(unsigned W) {
+    switch (W) {
+        case 1: return ScatterShape<1>::NT;
+        case 2: return ScatterShape<2>::NT;
+        case 3: return ScatterShape<3>::NT;
+        default: return ScatterShape<4>::NT;
+    }
 }
 
 size_t scatter_smem_bytes(unsigned W, unsigned p1) {
@@ -114,7 +136,7 @@ static cudaError_t launch_scatter_wpg(const Job* jobs, const unsigned long long*
     if (e != cudaSuccess) return e;
     if (tiles == 0) return cudaSuccess;
     if (tiles > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    scatter_kernel<W, MAXPER, HI, GATE><<<(unsigned)tiles, kStageThreads, smem, s>>>(jobs, tile_off, n_jobs);
+    scatter_kernel<W, MAXPER, HI, GATE><<<(unsigned)tiles, ScatterShape<W>::NT, smem, s>>>(jobs, tile_off, n_jobs);
     return cudaGetLastError();
 }
 
@@ -128,12 +150,14 @@ static cudaError_t launch_scatter_wp(const Job* jobs, const unsigned long long* 
 template <int W, bool HI>
 static cudaError_t launch_scatter_w(const Job* jobs, const unsigned long long* tile_off, unsigned n_jobs,
                                     unsigned long long tiles, unsigned max_p1, bool gated, cudaStream_t s) {
-    // MAXPER: destinations of one thread in a flush (fan-out / 256, rounded up to 2, 4 or 8)
-    if ((1u << max_p1) <= 2 * kStageThreads)
+    // MAXPER: destinations of one thread in a flush (fan-out / threads, rounded up)
+    constexpr unsigned NT = ScatterShape<W>::NT;
+    if ((1u << max_p1) <= 2 * NT)
         return launch_scatter_wp<W, 2, HI>(jobs, tile_off, n_jobs, tiles, max_p1, gated, s);
-    if ((1u << max_p1) <= 4 * kStageThreads)
-        return launch_scatter_wp<W, 4, HI>(jobs, tile_off, n_jobs, tiles, max_p1, gated, s);
-    return launch_scatter_wp<W, kMaxStageDest / kStageThreads, HI>(jobs, tile_off, n_jobs, tiles, max_p1, gated, s);
+    if constexpr (kMaxStageDest / NT > 4)
+        if ((1u << max_p1) <= 4 * NT)
+            return launch_scatter_wp<W, 4, HI>(jobs, tile_off, n_jobs, tiles, max_p1, gated, s);
+    return launch_scatter_wp<W, kMaxStageDest / NT, HI>(jobs, tile_off, n_jobs, tiles, max_p1, gated, s);
 }
 
 cudaError_t launch_scatter(unsigned W, const Job* jobs, const unsigned long long* tile_off, unsigned n_jobs,
