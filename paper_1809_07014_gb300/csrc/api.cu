@@ -122,6 +122,10 @@ Geometry plan_geometry(unsigned k, unsigned long long windows, unsigned long lon
     // ranges)
     const unsigned long long target = std::max(64ull, (unsigned long long)cap_max * 3 / 4);
     unsigned p = leaf_bits ? leaf_bits : ceil_log2((basis + target - 1) / target);
+    // small inputs: a leaf for most CTAs of the leaf kernel (256), of 512 windows
+    // or more (260 000 windows in 64 leaves left four of five CTAs idle)
+    if (!leaf_bits)
+        while (p < 8 && (windows >> (p + 1)) >= 512) ++p;
     const unsigned need = g.bt > 58 ? g.bt - 58 : 0;  // partition bits implied by the record format
     p = std::max(p, need);
     p = std::min(p, g.bt);
@@ -826,7 +830,9 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
             j.gate_bits = h->gate_bits;
         }
         // one scatter job per submitted readset, one CTA per tile of reads
-        const unsigned tile_reads = scatter_tile_reads(W);
+        unsigned long long all_reads = 0;
+        for (const kmer_readset* rs : h->submitted) all_reads += rs->n_reads;
+        const unsigned seg_bits = scatter_seg_bits(all_reads, h->num_sms), tile_reads = scatter_tile_reads(seg_bits);
         std::vector<Job> sjobs;
         std::vector<unsigned long long> tile_off(1, 0);
         for (const kmer_readset* rs : h->submitted) {
@@ -841,7 +847,7 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
         TRY(prof_begin(h, kmer_analysis::STG_SCATTER));
         if (!sjobs.empty()) {
             CK(launch_scatter(W, h->d_sjobs.as<Job>(), h->d_tile_off.as<unsigned long long>(), (unsigned)sjobs.size(),
-                              tile_off.back(), g.p1, g.k, j.gate != nullptr, h->stream));
+                              tile_off.back(), seg_bits, g.p1, g.k, j.gate != nullptr, h->stream));
             h->st.launches++;
         }
         TRY(prof_end(h, kmer_analysis::STG_SCATTER));

@@ -58,7 +58,7 @@ struct BJob {
 struct Wave {
     std::vector<unsigned> ids;  // job indices, grouped by key width
     struct Cls {
-        unsigned W, first, count, max_p1, max_p2, cap_max, min_k;
+        unsigned W, first, count, max_p1, max_p2, cap_max, min_k, seg_bits;
         unsigned long long tiles, leaves;
     };
     std::vector<Cls> classes;
@@ -210,7 +210,10 @@ int capture_wave(kmer_batch* b, Wave& w) {
     std::vector<unsigned long long> host_maps;
     for (auto& c : w.classes) {
         std::vector<unsigned long long> tile_off(1, 0), leaf_off(1, 0);
-        const unsigned tile_reads = scatter_tile_reads(c.W);
+        unsigned long long all_reads = 0;
+        for (unsigned i = 0; i < c.count; ++i) all_reads += b->jobs[w.ids[c.first + i]].rs->n_reads;
+        c.seg_bits = scatter_seg_bits(all_reads, b->num_sms);
+        const unsigned tile_reads = scatter_tile_reads(c.seg_bits);
         for (unsigned i = 0; i < c.count; ++i) {
             const BJob& j = b->jobs[w.ids[c.first + i]];
             tile_off.push_back(tile_off.back() + (j.rs->n_reads + tile_reads - 1) / tile_reads);
@@ -243,7 +246,7 @@ int capture_wave(kmer_batch* b, Wave& w) {
         if (e == cudaSuccess) e = cudaMemsetAsync(b->misc.as<Misc>() + id, 0, sizeof(Misc), b->stream);
     for (size_t ci = 0; ci < w.classes.size() && e == cudaSuccess; ++ci) {
         const auto& c = w.classes[ci];
-        e = launch_scatter(c.W, dj + c.first, maps + w.tile_off_at[ci], c.count, c.tiles, c.max_p1, c.min_k, false,
+        e = launch_scatter(c.W, dj + c.first, maps + w.tile_off_at[ci], c.count, c.tiles, c.seg_bits, c.max_p1, c.min_k, false,
                            b->stream);
     }
     for (size_t ci = 0; ci < w.classes.size() && e == cudaSuccess; ++ci) {

@@ -114,15 +114,17 @@ cudaError_t launch_sort_by_digits(unsigned W, unsigned long long* keys, unsigned
                                   unsigned char* cls, unsigned long long n, unsigned k, void* scratch,
                                   unsigned* status, int num_sms, unsigned* launches, cudaStream_t s);
 
-// Level-1 scatter (a2-a3 + partition): one CTA per tile of scatter_tile_reads(W) reads;
+// Level-1 scatter (a2-a3 + partition): one CTA per tile of scatter_tile_reads(seg_bits) reads;
 // tile_off = exclusive prefix (n_jobs + 1) of the jobs' read tiles; min_k =
 // the smallest k of the jobs (one-word keys with k >= 17 roll on their high
 // half).
 size_t scatter_smem_bytes(unsigned W, unsigned p1);
-unsigned scatter_tile_reads(unsigned W);  // reads of a tile
+unsigned scatter_seg_bits(unsigned long long n_reads, int num_sms);  // log2 of the threads that share a read
+unsigned scatter_tile_reads(unsigned seg_bits);                       // reads of a tile
 // gated: every job carries a Bloom gate (Job::gate) and emits only its keys.
 cudaError_t launch_scatter(unsigned W, const Job* jobs, const unsigned long long* tile_off, unsigned n_jobs,
-                           unsigned long long tiles, unsigned max_p1, unsigned min_k, bool gated, cudaStream_t s);
+                           unsigned long long tiles, unsigned seg_bits, unsigned max_p1, unsigned min_k, bool gated,
+                           cudaStream_t s);
 
 // Per analysis: level-2 tile counts, leaf capacities and leaf region bases;
 // then job_tile_off = prefix of the analyses' level-2 tiles (device array).

@@ -39,11 +39,11 @@ __device__ __forceinline__ unsigned long long revcomp_word(unsigned long long x)
     return ((m >> 1) & 0x5555555555555555ull) | ((m & 0x5555555555555555ull) << 1);
 }
 
-// One read's windows in order.  init() stands at the first window: its words
-// come from the packed blocks by shifts, its reverse complement by bit
-// reversal and the last N before it from the N masks, so the k bases of the
-// first window cost no steps (two thirds of a 150-base read's steps at
-// k = 99, a fifth at k = 31).
+// One read's windows in order, from any window on.  init() stands at window
+// w0: its words come from the packed blocks by shifts, its reverse complement
+// by bit reversal and the last N before it from the N masks, so the k bases
+// of the first window cost no steps (two thirds of a 150-base read's steps at
+// k = 99, a fifth at k = 31), and several threads can share a read.
 //
 // HI (one word, k >= 17): the window's first base sits in the high 32 bits
 // of the word, so the base leaving the window and the complement entering the
@@ -61,8 +61,9 @@ struct Roll {
     const PackedBlock* blk;
     unsigned long long mask;       // bits of word 0
 
-    // Stands before step k (reads shorter than k have no steps).
-    __device__ void init(const Job& j, unsigned long long r) {
+    // Stands before step k + w0, at the window of bases [w0, w0 + k); a read
+    // without that window (w0 + k > L) has no steps.
+    __device__ void init(const Job& j, unsigned long long r, unsigned w0 = 0) {
         const unsigned long long a = j.offsets[r];
         L = (unsigned)(j.offsets[r + 1] - a);  // reads are shorter than 2^31 bases
         blk = j.blocks + j.blk_off[r];
@@ -70,36 +71,58 @@ struct Roll {
         const unsigned hb = j.g.hb;
         mask = low_mask(hb);
         sh = hb - 2;
-        first_ok = k;
+        const unsigned t = w0 + k;
+        first_ok = t;
         out = lg = lgn = 0;
         cur = 0;
         curn = curg = 0;
         nxt = make_uint4(0, 0, 0, 0);
 #pragma unroll
         for (int i = 0; i < W; ++i) fwd[i] = rc[i] = 0;
-        if (L < k) return;
-        unsigned long long B[W];
-        unsigned last_n = 0;  // last N of the first k bases, plus one
-#pragma unroll
-        for (int i = 0; i < W; ++i) {  // k > 32 (W - 1): the first W blocks hold the first window
-            const uint4 x = __ldg(reinterpret_cast<const uint4*>(blk + i));
-            B[i] = (unsigned long long)x.y << 32 | x.x;
-            unsigned nm = x.z;
-            if (i == W - 1) {
-                const unsigned o = k - 32 * (W - 1);  // 1..31 bases of this block (k odd)
-                nm &= (1u << o) - 1u;
-                cur = B[i] << (2 * o);
-                curn = x.z >> o;
-                curg = x.w >> o;
-            }
-            if (nm) last_n = 32 * i + 32 - __clz(nm);
-            if (i == 0) lgn = x.w;
+        if (t > L) return;
+        // A[i]: the 32 bases from w0 + 32 i on, from two blocks (none past the read's last)
+        const unsigned b0 = w0 >> 5, o = w0 & 31u, o2 = 2 * o;
+        const unsigned blocks = (L + 31) / 32;
+        const uint4 none = make_uint4(0, 0, 0, 0);
+        uint4 x = __ldg(reinterpret_cast<const uint4*>(blk + b0));
+        if (o == 0) lgn = x.w;
+        else lg = x.w >> (o - 1);  // base w0 - 1 next
+        if (w0) {
+            const uint4 y = o ? x : __ldg(reinterpret_cast<const uint4*>(blk + b0 - 1));
+            if (!o) lg = y.w >> 31;
+            const unsigned at = (w0 - 1) & 31u;
+            out = (unsigned)((((unsigned long long)y.y << 32 | y.x) >> (62 - 2 * at)) & 3ull);
         }
-        if (last_n) first_ok = last_n + k;
-        if (32u * W < L) nxt = __ldg(reinterpret_cast<const uint4*>(blk + W));
-        fwd[0] = B[0] >> (64 - hb);
+        unsigned long long A[W];
+        unsigned last_n = 0;  // last N of the window, plus one, from w0
+        const unsigned rest = k - 32 * (W - 1);  // 1..31 bases of the last word (k odd)
 #pragma unroll
-        for (int i = 1; i < W; ++i) fwd[i] = (B[i - 1] << hb) | (B[i] >> (64 - hb));
+        for (int i = 0; i < W; ++i) {
+            const bool more = b0 + i + 1 < blocks;
+            const uint4 y = more ? __ldg(reinterpret_cast<const uint4*>(blk + b0 + i + 1)) : none;
+            if (i == 0 && o) lgn = y.w;
+            const unsigned long long bx = (unsigned long long)x.y << 32 | x.x, by = (unsigned long long)y.y << 32 | y.x;
+            A[i] = o ? (bx << o2) | (by >> (64 - o2)) : bx;
+            unsigned nm = __funnelshift_r(x.z, y.z, o);
+            if (i == W - 1) nm &= (1u << rest) - 1u;
+            if (nm) last_n = 32 * i + 32 - __clz(nm);
+            if (i == W - 1) {  // base t is in this block or the next
+                const unsigned ot = t & 31u;
+                const bool same = t >> 5 == b0 + i;
+                const uint4 c = same ? x : y;
+                cur = ((unsigned long long)c.y << 32 | c.x) << (2 * ot);
+                curn = c.z >> ot;
+                curg = c.w >> ot;
+                // the block after base t's; step t takes nxt when t starts a block
+                const unsigned nb = ot ? (t >> 5) + 1 : t >> 5;
+                nxt = nb < blocks ? __ldg(reinterpret_cast<const uint4*>(blk + nb)) : none;
+            }
+            x = y;
+        }
+        if (last_n) first_ok = w0 + last_n + k;
+        fwd[0] = A[0] >> (64 - hb);
+#pragma unroll
+        for (int i = 1; i < W; ++i) fwd[i] = (A[i - 1] << hb) | (A[i] >> (64 - hb));
         unsigned long long R[W];
 #pragma unroll
         for (int i = 0; i < W; ++i) R[i] = revcomp_word(fwd[W - 1 - i]);
@@ -108,7 +131,7 @@ struct Roll {
         for (int i = 1; i < W; ++i) rc[i] = (R[i - 1] << hb) | (R[i] >> (64 - hb));
     }
 
-    // Step t = k, k + 1, ..., L, in order.  First the window [t-k, t) is
+    // Step t = w0 + k, w0 + k + 1, ..., L, in order.  First the window [t-k, t) is
     // reported if it holds no N; then base t (if t < L) is shifted in.
     // Returns true and fills key / lcode / rcode (0 = none, 1..4 = A..T) for a
     // window.
