@@ -1517,55 +1517,72 @@ int kmer_analysis_merge_contigs(kmer_analysis_t* h, const char* contigs, const u
         // piece's edge may come twice, once without the base beyond the edge,
         // which adds no base to its sides, and counts are not used.
         const unsigned long long kMergePiece = std::max<unsigned long long>(1024, 16ull * (h->p.k + 1));
-        std::vector<unsigned long long> off(n_contigs + 1);
-        if (where == KMER_DEVICE) {
-            CK(cudaMemcpyAsync(off.data(), offsets, off.size() * 8, cudaMemcpyDeviceToHost, h->stream));
-            CK(cudaStreamSynchronize(h->stream));
-        } else {
-            std::memcpy(off.data(), offsets, off.size() * 8);
-        }
-        std::vector<unsigned long long> psrc, pdst(1, 0);
-        bool cut = false;
-        for (uint64_t c = 0; c < n_contigs; ++c) {
-            const unsigned long long a = off[c], e = off[c + 1];
-            if (e < a) return fail(KMER_ERR_INVALID_ARG, "contig offsets decrease at %llu", (unsigned long long)c);
-            cut |= e - a > kMergePiece;
-            for (unsigned long long st = a;;) {
-                const unsigned long long en = std::min(e, st + kMergePiece);
-                psrc.push_back(st);
-                pdst.push_back(pdst.back() + (en - st));
-                if (en >= e) break;
-                st = en - (h->p.k + 1);
-            }
-        }
-        DevBuf d_pieces, d_psrc, d_pdst;
+        const unsigned long long kLap = h->p.k + 1;
+        DevBuf d_pieces, d_psrc, d_pdst, d_cut;
         std::vector<char> h_pieces;
+        std::vector<unsigned long long> psrc, pdst(1, 0);
         const char* cseq = contigs;
         const uint64_t* coff = offsets;
         uint64_t n_seq = n_contigs;
         int cwhere = where;
-        if (cut) {
-            const unsigned long long n_p = psrc.size(), bytes = pdst.back();
-            if (where == KMER_DEVICE) {
-                TRY(d_pieces.ensure(bytes + 16));
-                TRY(d_psrc.ensure(n_p * 8));
-                TRY(d_pdst.ensure((n_p + 1) * 8));
-                CK(cudaMemcpyAsync(d_psrc.p, psrc.data(), n_p * 8, cudaMemcpyHostToDevice, h->stream));
-                CK(cudaMemcpyAsync(d_pdst.p, pdst.data(), (n_p + 1) * 8, cudaMemcpyHostToDevice, h->stream));
-                CK(launch_piece_copy(contigs, d_psrc.as<unsigned long long>(), d_pdst.as<unsigned long long>(), n_p,
+        if (where == KMER_DEVICE) {
+            // counted, scanned and filled on the device: a loop over a million contigs
+            // on the host, and their offsets over the link, would leave the GPU idle
+            const unsigned long long* off = reinterpret_cast<const unsigned long long*>(offsets);
+            const size_t col = ((n_contigs + 2) * 8 + 255) & ~size_t(255);  // a scan also writes its total
+            TRY(d_cut.ensure(4 * col + 256 + scan_temp_bytes(n_contigs + 1)));
+            auto column = [&](int i) { return reinterpret_cast<unsigned long long*>(d_cut.as<char>() + i * col); };
+            unsigned long long *count = column(0), *bytes = column(1), *pstart = column(2), *bstart = column(3);
+            unsigned long long* bad = column(4);
+            void* temp = d_cut.as<char>() + 4 * col + 256;
+            CK(cudaMemsetAsync(bad, 0, 8, h->stream));
+            CK(launch_piece_count(off, n_contigs, kMergePiece, kLap, count, bytes, bad, h->num_sms, h->stream));
+            CK(exclusive_scan_u64(count, pstart, n_contigs, temp, h->stream));
+            CK(exclusive_scan_u64(bytes, bstart, n_contigs, temp, h->stream));
+            CK(cudaMemcpyAsync(bad + 1, pstart + n_contigs, 8, cudaMemcpyDeviceToDevice, h->stream));
+            CK(cudaMemcpyAsync(bad + 2, bstart + n_contigs, 8, cudaMemcpyDeviceToDevice, h->stream));
+            unsigned long long tot[3] = {0, 0, 0};  // contigs with decreasing offsets, pieces, bases
+            CK(cudaMemcpyAsync(tot, bad, sizeof tot, cudaMemcpyDeviceToHost, h->stream));
+            CK(cudaStreamSynchronize(h->stream));
+            h->st.launches += 7;
+            if (tot[0]) return fail(KMER_ERR_INVALID_ARG, "the offsets of %llu contigs decrease", tot[0]);
+            if (tot[1] != n_contigs) {  // some contig is cut
+                TRY(d_pieces.ensure(tot[2] + 16));
+                TRY(d_psrc.ensure(tot[1] * 8));
+                TRY(d_pdst.ensure((tot[1] + 1) * 8));
+                CK(launch_piece_fill(off, n_contigs, kMergePiece, kLap, pstart, bstart, tot[1],
+                                     d_psrc.as<unsigned long long>(), d_pdst.as<unsigned long long>(), h->num_sms,
+                                     h->stream));
+                CK(launch_piece_copy(contigs, d_psrc.as<unsigned long long>(), d_pdst.as<unsigned long long>(), tot[1],
                                      d_pieces.as<char>(), h->num_sms, h->stream));
-                h->st.launches++;
+                h->st.launches += 2;
                 cseq = d_pieces.as<char>();
                 coff = reinterpret_cast<const uint64_t*>(d_pdst.p);
-            } else {
-                h_pieces.resize(bytes);
-                for (unsigned long long i = 0; i < n_p; ++i)
+                n_seq = tot[1];
+            }
+        } else {
+            bool cut = false;
+            for (uint64_t c = 0; c < n_contigs; ++c) {
+                const unsigned long long a = offsets[c], e = offsets[c + 1];
+                if (e < a) return fail(KMER_ERR_INVALID_ARG, "contig offsets decrease at %llu", (unsigned long long)c);
+                cut |= e - a > kMergePiece;
+                for (unsigned long long st = a;;) {
+                    const unsigned long long en = std::min<unsigned long long>(e, st + kMergePiece);
+                    psrc.push_back(st);
+                    pdst.push_back(pdst.back() + (en - st));
+                    if (en >= e) break;
+                    st = en - kLap;
+                }
+            }
+            if (cut) {
+                h_pieces.resize(pdst.back());
+                for (size_t i = 0; i < psrc.size(); ++i)
                     std::memcpy(h_pieces.data() + pdst[i], contigs + psrc[i], pdst[i + 1] - pdst[i]);
                 cseq = h_pieces.data();
                 coff = reinterpret_cast<const uint64_t*>(pdst.data());
                 cwhere = KMER_HOST_STAGED;
+                n_seq = psrc.size();
             }
-            n_seq = n_p;
         }
         kmer_readset_t* crs = nullptr;
         TRY(make_readset(cseq, reinterpret_cast<const uint8_t*>(cseq), coff, n_seq, 0, 0, cwhere, h->stream, &crs));

@@ -71,6 +71,15 @@ cudaError_t launch_gate(const Job& j, unsigned long long* f1, unsigned long long
 // bcls; bn of them) absent from the indexed survivors are appended to them
 // from position *n_out on (count 0, zero tallies, their own classes); a
 // position past out_cap sets bit 0 of *status.
+// Contigs cut into overlapping pieces (device offsets): pieces and bases of
+// each contig, then each piece's source and destination.
+cudaError_t launch_piece_count(const unsigned long long* off, unsigned long long n, unsigned long long piece,
+                               unsigned long long lap, unsigned long long* count, unsigned long long* bytes,
+                               unsigned long long* bad, int num_sms, cudaStream_t s);
+cudaError_t launch_piece_fill(const unsigned long long* off, unsigned long long n, unsigned long long piece,
+                              unsigned long long lap, const unsigned long long* pstart,
+                              const unsigned long long* bstart, unsigned long long n_pieces, unsigned long long* psrc,
+                              unsigned long long* pdst, int num_sms, cudaStream_t s);
 // Pieces of a byte string: piece i is src[psrc[i] ..) of pdst[i + 1] - pdst[i]
 // bytes, written to dst[pdst[i] ..) (pdst: n_pieces + 1 offsets).
 cudaError_t launch_piece_copy(const char* src, const unsigned long long* psrc, const unsigned long long* pdst,

@@ -71,12 +71,22 @@ __device__ __forceinline__ void shift_in_left(unsigned long long (&x)[W], unsign
     x[0] = (x[0] >> 2) | ((unsigned long long)b << (hb - 2));
 }
 
+// Whole words: the bases of each reversed and complemented by bit reversal,
+// then all moved down by the unused bits of word 0 (which uses hb, 2 to 62 for
+// odd k).
 template <int W>
 __device__ __forceinline__ void reverse_complement(const unsigned long long (&x)[W], unsigned k,
                                                    unsigned long long (&rc)[W]) {
+    const unsigned hb = 2 * k - 64 * (W - 1);
+    unsigned long long r[W];
 #pragma unroll
-    for (int w = 0; w < W; ++w) rc[w] = 0;
-    for (unsigned b = 0; b < k; ++b) set_base<W>(rc, k, k - 1 - b, 3u - get_base<W>(x, k, b));
+    for (int w = 0; w < W; ++w) {
+        const unsigned long long m = __brevll(~x[W - 1 - w]);
+        r[w] = ((m >> 1) & 0x5555555555555555ull) | ((m & 0x5555555555555555ull) << 1);
+    }
+    rc[0] = r[0] >> (64 - hb);
+#pragma unroll
+    for (int w = 1; w < W; ++w) rc[w] = (r[w - 1] << hb) | (r[w] >> (64 - hb));
 }
 
 // a < b, word 0 first (lexicographic order of the k-mers).

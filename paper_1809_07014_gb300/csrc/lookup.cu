@@ -40,14 +40,11 @@ __global__ void __launch_bounds__(256) lookup_kernel(const unsigned long long* _
     for (unsigned long long i = blockIdx.x * 256ull + threadIdx.x; i < n; i += (unsigned long long)gridDim.x * 256) {
         unsigned long long key[W], rc[W];
 #pragma unroll
-        for (int w = 0; w < W; ++w) {
-            key[w] = q[i * W + w];
-            rc[w] = 0;
-        }
+        for (int w = 0; w < W; ++w) key[w] = q[i * W + w];
         kmer_record r{};
         const bool valid = hb >= 64 || (key[0] >> hb) == 0ull;  // no bits above 2k
         if (valid) {
-            for (unsigned b = 0; b < k; ++b) set_base<W>(rc, k, k - 1 - b, 3u - get_base<W>(key, k, b));
+            reverse_complement<W>(key, k, rc);
             bool flip = false;
 #pragma unroll
             for (int w = 0; w < W; ++w) {
@@ -163,6 +160,69 @@ cudaError_t launch_index_build(unsigned W, const unsigned long long* keys, unsig
         case 4: index_build_kernel<4><<<g, 256, 0, s>>>(keys, n, idx, cap); break;
         default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
+}
+
+// Cutting of contigs into pieces of `piece` bases that overlap by `lap`: a
+// contig of L bases gives 1 + ceil((L - piece) / (piece - lap)) pieces (one if
+// L <= piece), every one but the last of `piece` bases.
+// count[c], bytes[c]: pieces of contig c and their bases; *bad counts
+// contigs whose offsets decrease.
+__global__ void __launch_bounds__(256) piece_count_kernel(const unsigned long long* __restrict__ off,
+                                                          unsigned long long n, unsigned long long piece,
+                                                          unsigned long long lap, unsigned long long* __restrict__ count,
+                                                          unsigned long long* __restrict__ bytes,
+                                                          unsigned long long* __restrict__ bad) {
+    for (unsigned long long c = blockIdx.x * 256ull + threadIdx.x; c < n; c += (unsigned long long)gridDim.x * 256) {
+        const unsigned long long a = off[c], e = off[c + 1];
+        if (e < a) {
+            atomicAdd(bad, 1ull);
+            count[c] = bytes[c] = 0;
+            continue;
+        }
+        const unsigned long long L = e - a, extra = L > piece ? (L - piece + (piece - lap) - 1) / (piece - lap) : 0ull;
+        count[c] = extra + 1;
+        bytes[c] = L + extra * lap;
+    }
+}
+
+// Source and destination of every piece, from the scanned counts (pstart) and
+// bases (bstart): n_pieces threads, each finding its contig by binary search.
+__global__ void __launch_bounds__(256) piece_fill_kernel(const unsigned long long* __restrict__ off,
+                                                         unsigned long long n, unsigned long long piece,
+                                                         unsigned long long lap,
+                                                         const unsigned long long* __restrict__ pstart,
+                                                         const unsigned long long* __restrict__ bstart,
+                                                         unsigned long long n_pieces,
+                                                         unsigned long long* __restrict__ psrc,
+                                                         unsigned long long* __restrict__ pdst) {
+    for (unsigned long long p = blockIdx.x * 256ull + threadIdx.x; p < n_pieces; p += (unsigned long long)gridDim.x * 256) {
+        unsigned long long lo = 0, hi = n;  // pstart[lo] <= p < pstart[hi]
+        while (hi - lo > 1) {
+            const unsigned long long mid = (lo + hi) / 2;
+            if (pstart[mid] <= p) lo = mid; else hi = mid;
+        }
+        const unsigned long long i = p - pstart[lo];
+        psrc[p] = off[lo] + i * (piece - lap);
+        pdst[p] = bstart[lo] + i * piece;
+        if (p == n_pieces - 1) pdst[n_pieces] = bstart[n];
+    }
+}
+
+cudaError_t launch_piece_count(const unsigned long long* off, unsigned long long n, unsigned long long piece,
+                               unsigned long long lap, unsigned long long* count, unsigned long long* bytes,
+                               unsigned long long* bad, int num_sms, cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    piece_count_kernel<<<grid_of(n, num_sms), 256, 0, s>>>(off, n, piece, lap, count, bytes, bad);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_piece_fill(const unsigned long long* off, unsigned long long n, unsigned long long piece,
+                              unsigned long long lap, const unsigned long long* pstart,
+                              const unsigned long long* bstart, unsigned long long n_pieces, unsigned long long* psrc,
+                              unsigned long long* pdst, int num_sms, cudaStream_t s) {
+    if (n_pieces == 0) return cudaSuccess;
+    piece_fill_kernel<<<grid_of(n_pieces, num_sms), 256, 0, s>>>(off, n, piece, lap, pstart, bstart, n_pieces, psrc, pdst);
     return cudaGetLastError();
 }
 

@@ -158,67 +158,101 @@ __global__ void __launch_bounds__(256) walk_jump_kernel(unsigned long long* wk, 
 // Rulers: one port in 16 by a hash of its code, and every path start.
 __device__ __forceinline__ bool sampled_port(unsigned P) { return ((P * 2654435761u) >> 28) == 0u; }
 
-// Every ruler walks to the next ruler or to its path's end: owner[V] and
-// off[V] of each port V it passes (itself included) name it and V's distance
-// from it; rw[R] = (next ruler or end port, steps), and rw[E] = (E, 0) for
-// every end port E.  Rulers that have not reached an end go to the active
-// list.  Ports on rings without a ruler keep owner kNoPort.  A walk is
-// bounded by the number of ports (it cannot be longer unless the links were
-// not mutual), and one that gives up is counted in *err.
-__global__ void __launch_bounds__(256) ruler_walk_kernel(const unsigned* __restrict__ link, unsigned long long ports,
-                                                         unsigned* __restrict__ owner, unsigned* __restrict__ off,
+// Per vertex: own[P] = P at distance 0 for the rulers among its two ports, all
+// ones for the others (a port on a ring without a ruler keeps that); rw[E] =
+// (E, 0) for every end port E; the rulers with a partner are listed in act.  A
+// warp takes 256 vertices and adds their rulers with one atomic (two per 32
+// vertices made 1 M atomics on one address: 0.69 ms for 17 M vertices, under
+// 0.14 this way).
+__global__ void __launch_bounds__(256) ruler_list_kernel(const uint2* __restrict__ link, unsigned long long n,
+                                                         ulonglong2* __restrict__ own,
                                                          unsigned long long* __restrict__ rw, unsigned* act,
-                                                         unsigned* cnt, unsigned* err) {
-    for (unsigned long long P64 = blockIdx.x * 256ull + threadIdx.x; P64 < ports;
-         P64 += (unsigned long long)gridDim.x * 256) {
-        const unsigned P = (unsigned)P64;
-        const unsigned L = link[P];
-        if (L == kNoPort) rw[P] = walk_pack(P, 0u);
-        const bool ruler = link[P ^ 1u] == kNoPort || sampled_port(P);  // a path start has no predecessor
-        bool active = false;
-        if (ruler) {
-            owner[P] = P;
-            off[P] = 0;
-            if (L != kNoPort) {
-                unsigned cur = L ^ 1u, steps = 1;
-                for (;;) {
-                    if (sampled_port(cur)) break;  // the next ruler (only path starts lack a predecessor)
-                    owner[cur] = P;
-                    off[cur] = steps;
-                    const unsigned nl = link[cur];
-                    if (nl == kNoPort) break;  // the path's end
-                    if (steps >= ports) {
-                        atomicAdd(err, 1u);
-                        break;
-                    }
-                    cur = nl ^ 1u;
-                    ++steps;
-                }
-                // either a ruler (its own walk continues from there) or an end port
-                rw[P] = walk_pack(cur, steps);
-                active = true;
+                                                         unsigned* cnt) {
+    constexpr int kSteps = 8;
+    const unsigned lane = threadIdx.x & 31u, before = (1u << lane) - 1u;
+    const unsigned long long warp = (blockIdx.x * 256ull + threadIdx.x) / 32, warps = (unsigned long long)gridDim.x * 8;
+    for (unsigned long long v0 = warp * 32 * kSteps; v0 < n; v0 += warps * 32 * kSteps) {
+        unsigned m0[kSteps], m1[kSteps], total = 0;
+#pragma unroll
+        for (int u = 0; u < kSteps; ++u) {
+            const unsigned long long i = v0 + 32 * u + lane;
+            bool a0 = false, a1 = false;
+            if (i < n) {
+                const uint2 L = link[i];
+                const unsigned P = 2u * (unsigned)i, Q = P + 1u;
+                if (L.x == kNoPort) rw[P] = walk_pack(P, 0u);
+                if (L.y == kNoPort) rw[Q] = walk_pack(Q, 0u);
+                const bool r0 = L.y == kNoPort || sampled_port(P);  // a path start has no predecessor
+                const bool r1 = L.x == kNoPort || sampled_port(Q);
+                own[i] = make_ulonglong2(r0 ? walk_pack(P, 0u) : ~0ull, r1 ? walk_pack(Q, 0u) : ~0ull);
+                a0 = r0 && L.x != kNoPort;
+                a1 = r1 && L.y != kNoPort;
             }
+            m0[u] = __ballot_sync(0xffffffffu, a0);
+            m1[u] = __ballot_sync(0xffffffffu, a1);
+            total += __popc(m0[u]) + __popc(m1[u]);
         }
-        append_if(active, P, act, cnt);
+        unsigned base = 0;
+        if (lane == 0 && total) base = atomicAdd(cnt, total);
+        base = __shfl_sync(0xffffffffu, base, 0);
+#pragma unroll
+        for (int u = 0; u < kSteps; ++u) {
+            const unsigned P = 2u * (unsigned)(v0 + 32 * u + lane);
+            if (m0[u] >> lane & 1u) act[base + __popc(m0[u] & before)] = P;
+            base += __popc(m0[u]);
+            if (m1[u] >> lane & 1u) act[base + __popc(m1[u] & before)] = P + 1u;
+            base += __popc(m1[u]);
+        }
+    }
+}
+
+// Every listed ruler walks to the next ruler or to its path's end: own[V] =
+// (the ruler, V's distance from it) for each port V it passes, rw[R] = (next
+// ruler or end port, steps).  One ruler per thread of a full warp (walks from
+// the ports themselves left 30 of 32 lanes waiting: 2.4-2.9 ms for 33 M ports,
+// 1.3-1.6 this way), so the walks' dependent loads overlap.  A walk is bounded
+// by the number of ports (it cannot be longer unless the links were not
+// mutual), and one that gives up is counted in *err.
+__global__ void __launch_bounds__(256) ruler_walk_kernel(const unsigned* __restrict__ link, unsigned long long ports,
+                                                         const unsigned* __restrict__ act,
+                                                         const unsigned* __restrict__ cnt,
+                                                         unsigned long long* __restrict__ own,
+                                                         unsigned long long* __restrict__ rw, unsigned* err) {
+    const unsigned n = *cnt;
+    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) {
+        const unsigned P = act[i];
+        unsigned cur = link[P] ^ 1u, steps = 1;
+        while (!sampled_port(cur)) {  // else the next ruler (only path starts lack a predecessor)
+            own[cur] = walk_pack(P, steps);
+            const unsigned nl = link[cur];
+            if (nl == kNoPort) break;  // the path's end
+            if (steps >= ports) {
+                atomicAdd(err, 1u);
+                break;
+            }
+            cur = nl ^ 1u;
+            ++steps;
+        }
+        // either a ruler (its own walk continues from there) or an end port
+        rw[P] = walk_pack(cur, steps);
     }
 }
 
 // Every port's walk from its ruler's: the same end, less the distance from
 // the ruler; ports on rings get cap_dist.
 __global__ void __launch_bounds__(256) ruler_final_kernel(const unsigned* __restrict__ link, unsigned long long ports,
-                                                          const unsigned* __restrict__ owner,
-                                                          const unsigned* __restrict__ off,
+                                                          const unsigned long long* __restrict__ own,
                                                           const unsigned long long* __restrict__ rw, unsigned cap_dist,
                                                           unsigned long long* __restrict__ wk) {
     for (unsigned long long P = blockIdx.x * 256ull + threadIdx.x; P < ports; P += (unsigned long long)gridDim.x * 256) {
-        const unsigned R = owner[P];
-        if (R == kNoPort) {  // a ring with no ruler
+        const unsigned long long o = own[P];
+        if (o == ~0ull) {  // a ring with no ruler
             wk[P] = walk_pack(link[P] ^ 1u, cap_dist);
             continue;
         }
-        const unsigned long long w = rw[R];
+        const unsigned long long w = rw[walk_at(o)];
         const unsigned d = walk_dist(w);
-        wk[P] = d >= cap_dist ? walk_pack(walk_at(w), cap_dist) : walk_pack(walk_at(w), d - off[P]);
+        wk[P] = d >= cap_dist ? walk_pack(walk_at(w), cap_dist) : walk_pack(walk_at(w), d - walk_dist(o));
     }
 }
 
@@ -541,13 +575,13 @@ cudaError_t launch_traverse_plan(unsigned W, const unsigned long long* keys, con
         case 4: links_kernel<4><<<g, 256, 0, s>>>(keys, cls, n, k, idx, cap, t.link); break;
         default: return cudaErrorInvalidValue;
     }
-    // list ranking of every port by a ruling set (owners and distances in
-    // ra / rb, the rulers' walks in sa: all free until the rings are found)
-    e = cudaMemsetAsync(t.ra, 0xFF, 4 * ports, s);
-    if (e != cudaSuccess) return e;
-    ruler_walk_kernel<<<gp, 256, 0, s>>>(t.link, ports, t.ra, t.rb, t.sa, t.act_a, cnt_rank, walk_err);
+    // list ranking of every port by a ruling set (ports' rulers in sb, the
+    // rulers' walks in sa: both free until the rings are found)
+    ruler_list_kernel<<<g, 256, 0, s>>>(reinterpret_cast<const uint2*>(t.link), n, reinterpret_cast<ulonglong2*>(t.sb),
+                                        t.sa, t.act_a, cnt_rank);
+    ruler_walk_kernel<<<gp, 256, 0, s>>>(t.link, ports, t.act_a, cnt_rank, t.sb, t.sa, walk_err);
     jump_rounds(t, t.sa, cnt_rank, rounds, cap_dist, num_sms, s);
-    ruler_final_kernel<<<gp, 256, 0, s>>>(t.link, ports, t.ra, t.rb, t.sa, cap_dist, t.wk);
+    ruler_final_kernel<<<gp, 256, 0, s>>>(t.link, ports, t.sb, t.sa, cap_dist, t.wk);
     // rings: the smallest vertex of each, cut before it, and their ports ranked again
     ring_init_kernel<<<gp, 256, 0, s>>>(t.wk, ports, cap_dist, t.link, t.ra, t.sa, t.ring, ring_n);
     unsigned n_ring = 0, n_err = 0;
