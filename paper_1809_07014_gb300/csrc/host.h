@@ -23,6 +23,14 @@ cudaError_t launch_lookup(unsigned W, const unsigned long long* q, unsigned long
                           const unsigned* count, const unsigned* ext, const unsigned char* cls, kmer_record* out,
                           int num_sms, cudaStream_t s);
 
+// The same without an index: the n keys go into a table in `scratch`
+// (wanted_scratch_bytes) and the n_out survivors stream past it once.
+size_t wanted_scratch_bytes(unsigned W, unsigned long long n);
+cudaError_t launch_wanted(unsigned W, const unsigned long long* q, unsigned long long n, unsigned k, void* scratch,
+                          const unsigned long long* keys, const unsigned* count, const unsigned* ext,
+                          const unsigned char* cls, unsigned long long n_out, kmer_record* out, int num_sms,
+                          cudaStream_t s);
+
 // Records `code` with a formatted detail for kmer_last_error_message().
 int fail(int code, const char* fmt, ...);
 const char* last_error_message();

@@ -58,8 +58,8 @@ __host__ __device__ inline unsigned fallback_rs(unsigned e) { return e >> (kFbLe
 
 // Index of the survivors (positions in an open-addressing table of `cap`
 // slots, all 0xFFFFFFFF before the build) for point lookups (lookup.cu).
-cudaError_t launch_index_build(unsigned W, const unsigned long long* keys, unsigned long long n, unsigned* idx,
-                               unsigned long long cap, int num_sms, cudaStream_t s);
+cudaError_t launch_index_build(unsigned W, const unsigned long long* keys, unsigned long long n, unsigned k,
+                               unsigned* idx, unsigned long long cap, int num_sms, cudaStream_t s);
 
 // Bloom gate (gate.cu): adds every window's key of the job's reads to filter
 // f1, and keys already in f1 to f2 (both 2^log2_words words, zeroed by the
@@ -85,7 +85,7 @@ cudaError_t launch_piece_fill(const unsigned long long* off, unsigned long long 
 cudaError_t launch_piece_copy(const char* src, const unsigned long long* psrc, const unsigned long long* pdst,
                               unsigned long long n_pieces, char* dst, int num_sms, cudaStream_t s);
 cudaError_t launch_merge_append(unsigned W, const unsigned long long* bkeys, const unsigned char* bcls,
-                                unsigned long long bn, const unsigned* idx, unsigned long long cap,
+                                unsigned long long bn, unsigned k, const unsigned* idx, unsigned long long cap,
                                 unsigned long long* keys, unsigned* count, unsigned* ext, unsigned char* cls,
                                 unsigned long long out_cap, unsigned long long* n_out, unsigned* status, int num_sms,
                                 cudaStream_t s);

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(256) links_kernel(const unsigned long long* __
                     shift_in_right<W>(yr, 3u - b, hb);
                 }
                 const bool flip = key_less<W>(yr, y);
-                const unsigned j = index_find<W>(flip ? yr : y, idx, cap, keys);
+                const unsigned j = index_find<W>(flip ? yr : y, k, idx, cap, keys);
                 if (j == kIdxEmpty || j == i || !is_vertex(cls, j)) continue;
                 // y's base on the side facing x, read in y's orientation
                 bool mutual;
