@@ -207,6 +207,7 @@ struct kmer_analysis {
     // level-2 leaf slack (grown whenever a leaf overflowed)
     unsigned hist_k = 0;
     double hist_ratio = 0.0;
+    double rec_ratio = 0.0;  // distinct / records emitted at hist_k (fewer than the windows behind a Bloom gate)
     unsigned l2_slack_num = 512;  // leaf capacity = 2 * mean + 256
     double hint_ratio = 0.0;      // distinct_hint / windows of the current query (0 = no hint)
     // Bloom gate: filter words (log2), and first sightings / windows at hist_k
@@ -534,7 +535,7 @@ void fill_job_outputs(kmer_analysis* h, Job& j) {
     j.l2_slack_num = h->l2_slack_num;
     // leaf table: twice the expected distinct keys of a leaf (one slot per record if unknown)
     double ratio = 1.0;
-    if (h->hist_k == h->p.k && h->hist_ratio > 0.0) ratio = std::min(1.0, 2.0 * h->hist_ratio + 0.05);
+    if (h->hist_k == h->p.k && h->rec_ratio > 0.0) ratio = std::min(1.0, 2.0 * h->rec_ratio + 0.05);
     else if (h->hint_ratio > 0.0) ratio = std::min(1.0, 2.0 * h->hint_ratio + 0.05);
     j.table_ratio_num = (unsigned)(ratio * 65536.0);
 }
@@ -1128,6 +1129,7 @@ int do_query(kmer_analysis* h) {
     if (h->res_windows) {
         h->hist_k = h->p.k;
         h->hist_ratio = (double)h->res_distinct / (double)h->res_windows;
+        h->rec_ratio = (double)h->res_distinct / (double)std::max<uint64_t>(1, h->st.records_emitted);
     }
     h->st.windows = h->res_windows;
     h->st.distinct = h->res_distinct;

@@ -159,7 +159,7 @@ struct Job {
     // classification
     unsigned min_count, ext_mode, t_base, err_num, err_den, t_ext;
     // sizing: level-2 leaf capacity = mean * l2_slack_num / 256 + 256 records;
-    // leaf table slots = records * table_ratio_num / 65536 + 512 (capped)
+    // leaf table slots = records * table_ratio_num / 65536 + 1024 (capped)
     unsigned l2_slack_num;
     unsigned table_ratio_num;
     // status and statistics

@@ -24,12 +24,13 @@
 // What bounds it: latency of the probe rounds and the issue slots (about 0.67
 // instructions a cycle and scheduler, half of the shared-memory pipe), not
 // DRAM.  On the 2-Gbase reads at k = 31 (1.6 G records, 508 M keys) 18.5 ->
-// 14.4 ms, at k = 99 (103 M records, 89 M keys) 5.3 -> 3.7 ms, from: the
+// 13.6 ms, at k = 99 (103 M records, 89 M keys) 5.3 -> 3.7 ms, from: the
 // claiming record keeping its extension code in the slot (no tally for a third
 // of the records at k = 31, for six in seven at k = 99; most k-mers are seen
 // once), hashed steps between groups (consecutive groups clustered: leaves
 // above 0.6 of a table overflowed their probe limit), 32-bit shared-memory
-// addresses, job fields in shared memory instead of global loads in the sweep,
+// addresses, one-word probe rounds of full warps (a queue per warp: 14.4 ->
+// 13.6 ms), job fields in shared memory instead of global loads in the sweep,
 // four slots per lane in the sweep, and fuller leaves (0.75 of a table).
 //
 // Every plane is zero between leaves: the sweep clears each slot after
@@ -58,14 +59,19 @@ struct LeafShape {
     static constexpr int B = U * kLeafThreads;
 };
 
-// bytes per slot: tail, heads, 5 tally planes, survivor list entry
-__host__ __device__ inline size_t leaf_slot_bytes(unsigned W) { return (size_t)8 * W + 4 * kLanePlanes + 4; }
+// One-word records that a probe round leaves unsettled wait in their warp's
+// queue (the record and its probe state): up to 31 from before plus 32.
+constexpr unsigned kQueue = 64;
+__host__ __device__ inline size_t leaf_queue_bytes(unsigned W) { return W == 1 ? (size_t)kLeafWarps * kQueue * 12 : 0; }
 
-size_t leaf_smem_bytes(unsigned W, unsigned cap) { return leaf_slot_bytes(W) * cap + 64; }
+// bytes per slot: tail, heads, 5 tally planes, survivor list entry
+__host__ __device__ inline size_t leaf_slot_bytes(unsigned W) { return (size_t)8 * W + 4 * kLanePlanes + 2; }
+
+size_t leaf_smem_bytes(unsigned W, unsigned cap) { return leaf_slot_bytes(W) * cap + leaf_queue_bytes(W) + 64; }
 
 unsigned leaf_table_cap(unsigned W, size_t smem_budget) {
-    size_t c = (smem_budget - 64) / leaf_slot_bytes(W);
-    return (unsigned)(c & ~511ull);  // a whole number of warp slices of 32 slots
+    size_t c = (smem_budget - 64 - leaf_queue_bytes(W)) / leaf_slot_bytes(W);
+    return (unsigned)(c & ~63ull);  // a slice of a multiple of four slots per warp
 }
 
 struct LeafInfo {
@@ -122,7 +128,8 @@ struct Table {
     unsigned tail;    // 8 bytes a slot (two-word keys: 16, tail and head)
     unsigned heads;   // W - 1 planes of 8 bytes a slot
     unsigned lanes;   // 5 planes of 4 bytes a slot
-    unsigned list;    // 4 bytes a slot
+    unsigned list;    // 2 bytes a slot
+    unsigned queue;   // this warp's queue (one-word keys): kQueue records, then kQueue states
     unsigned stride;  // slots of a plane
 };
 
@@ -144,6 +151,14 @@ __device__ __forceinline__ uint4 lds128(unsigned a) {
 }
 __device__ __forceinline__ void sts32(unsigned a, unsigned v) {
     asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned lds16(unsigned a) {
+    unsigned short v;
+    asm volatile("ld.volatile.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts16(unsigned a, unsigned v) {
+    asm volatile("st.volatile.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
 }
 __device__ __forceinline__ void sts64(unsigned a, unsigned long long v) {
     asm volatile("st.volatile.shared.u64 [%0], %1;" ::"r"(a), "l"(v) : "memory");
@@ -202,28 +217,95 @@ __device__ __forceinline__ bool same_tail(unsigned lo, unsigned hi, unsigned klo
     return (((lo ^ klo) & ~63u) | (hi ^ khi)) == 0u && lo != 0u;
 }
 
-// Slot of a record's key, or kClaimed when the record claimed a new one,
-// kNoSlot after kMaxRounds full groups, kGaveUp after a wait that gave up.
-//
 // A key goes through groups home, home + step, ... of the table.  The slots of
 // a group fill in order and none empties while a leaf is counted, so a group's
 // first empty slot is the number of occupied ones, and a claim there can only
 // succeed when every slot before it holds a key that was compared: a key never
-// gets two slots.  Each round of the loop is one 16-byte load and at most one
-// claim.
+// gets two slots.  The record that claims a slot leaves its extension code
+// there; the others add to the slot's tallies.
 //
-// A lane leaves as soon as its record is settled and goes on to its next one
-// by itself.  The lanes of a warp drift apart that way, which pays: rounds are
-// latency (a load, a compare, a CAS), and lanes apart overlap theirs.
+// Home group from every in-leaf bit of z (the low bits of z depend on few
+// bits of the key, its top bits are the leaf's): a multiplicative hash.
+__device__ __forceinline__ unsigned leaf_hash(unsigned long long tail) {
+    return ((unsigned)tail & ~63u) * 0x9E3779B1u + (unsigned)(tail >> 32) * 0x85EBCA77u;
+}
+// Groups between one probe and the next: at least 256 groups, so that 64 steps never meet again.
+__device__ __forceinline__ unsigned leaf_step(unsigned hsh) { return (hsh >> 8 & 255u) | 1u; }
+
+__device__ __forceinline__ void tally(const Table& t, unsigned slot, unsigned long long tail) {
+    const unsigned l = ext_left(tail), r = ext_right(tail);
+    bump(t, slot, l ? l - 1 : 4u);  // every counted window has exactly one left lane (the first: its code)
+    if (r) bump(t, slot, 4u + r);
+}
+
+// One probe round of a warp (every lane calls; lanes with `have` hold a record
+// that probes group g, `full` groups so far): one 16-byte load, at most one
+// claim.  A record that is not settled (its group is full, or another key took
+// the slot it tried) goes to the warp's queue, `waiting` records so far.
+__device__ __forceinline__ void probe_round(const Table& t, const unsigned long long tail, bool have, unsigned g,
+                                            unsigned full, unsigned hsh, unsigned ngroups, unsigned& waiting,
+                                            unsigned* s_flags) {
+    // the code's + 1 does not carry out of bit 5
+    const unsigned klo = (unsigned)tail + 1u, khi = (unsigned)(tail >> 32);
+    bool again = false;
+    if (have) {
+        const unsigned ga = t.tail + 16 * g;
+        const uint4 a = lds128(ga);
+        const bool e0 = same_tail(a.x, a.y, klo, khi), e1 = same_tail(a.z, a.w, klo, khi);
+        bool hit = e0 || e1;
+        unsigned slot = 2 * g + (e1 ? 1u : 0u);
+        again = !hit;
+        if (!hit && a.z == 0u) {
+            const unsigned occ = a.x ? 1u : 0u;
+            const unsigned long long old = claim64(ga + 8 * occ, tail + 1ull);
+            slot = 2 * g + occ;
+            hit = old != 0ull && same_tail((unsigned)old, (unsigned)(old >> 32), klo, khi);
+            again = old != 0ull && !hit;  // another key took the slot: the group is read again
+        } else if (!hit) {
+            g += leaf_step(hsh);
+            g -= g >= ngroups ? ngroups : 0u;
+            ++full;
+        }
+        if (hit) tally(t, slot, tail);
+        if (full >= kMaxRounds) {
+            again = false;
+            atomicOr(s_flags, kLeafFull);
+        }
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, again);
+    if (again) {
+        const unsigned at = waiting + __popc(m & ((1u << (threadIdx.x & 31u)) - 1u));
+        sts64(t.queue + 8 * at, tail);
+        sts32(t.queue + 8 * kQueue + 4 * at, full << 16 | g);  // g is below 65 536
+    }
+    waiting += __popc(m);
+    __syncwarp();
+}
+
+// A probe round of the last (up to 32) records of the warp's queue.
+__device__ __forceinline__ void probe_queue(const Table& t, unsigned ngroups, unsigned& waiting, unsigned* s_flags) {
+    const unsigned n = waiting < 32u ? waiting : 32u, at = waiting - n + (threadIdx.x & 31u);
+    const bool have = (threadIdx.x & 31u) < n;
+    const unsigned long long tail = have ? lds64(t.queue + 8 * at) : 0ull;
+    const unsigned state = have ? lds32(t.queue + 8 * kQueue + 4 * at) : 0u;
+    __syncwarp();
+    waiting -= n;
+    probe_round(t, tail, have, state & 0xFFFFu, state >> 16, leaf_hash(tail), ngroups, waiting, s_flags);
+}
+
+// Two words and more: slot of a record's key, or kClaimed when the record
+// claimed a new one, kNoSlot after kMaxRounds full groups, kGaveUp after a
+// wait that gave up.  A lane leaves as soon as its record is settled: the
+// lanes of a warp drift apart, which pays here (queued full-warp rounds as for
+// one word, with either CAS, took 1.09 ms against 0.59 on 32 M two-word
+// records) and not there (20.5 ms against 14.3 on 1.6 G).
 constexpr int kClaimed = -1, kNoSlot = -2, kGaveUp = -3;
 
 template <int W>
 __device__ __forceinline__ int find_slot(const Table& t, const unsigned long long (&rec)[W], unsigned ngroups) {
     constexpr unsigned GS = W == 2 ? 1 : 2;  // slots of a group
-    // home group from every in-leaf bit of z (the low bits of z depend on few
-    // bits of the key, its top bits are the leaf's): a multiplicative hash
     const unsigned lo = (unsigned)rec[W - 1], khi = (unsigned)(rec[W - 1] >> 32), klo = lo + 1u;
-    const unsigned hsh = (lo & ~63u) * 0x9E3779B1u + khi * 0x85EBCA77u;
+    const unsigned hsh = leaf_hash(rec[W - 1]);
     const unsigned long long ktail = rec[W - 1] + 1ull;
     unsigned g = __umulhi(hsh, ngroups);
     for (unsigned it = 0; it < kMaxRounds;) {
@@ -263,70 +345,42 @@ __device__ __forceinline__ int find_slot(const Table& t, const unsigned long lon
             }
         }
         ++it;
-        g += (hsh >> 8 & 255u) | 1u;  // at least 256 groups: 64 steps never meet again
+        g += leaf_step(hsh);
         g -= g >= ngroups ? ngroups : 0u;
     }
     return kNoSlot;
 }
 
+// Counts one record per lane (lanes with `have`; every lane of the warp calls).
+//
+// One word: a first probe round, and a round of the queue whenever it
+// holds a full warp, so that every round has full warps (one record in seven
+// needs a second round at half a table; looping until the last lane is done
+// took two to three rounds with few lanes each).
 template <int W>
 __device__ __forceinline__ void count_record(const Table& t, const unsigned long long (&rec)[W], bool have,
-                                             unsigned ngroups, unsigned* s_flags) {
+                                             unsigned ngroups, unsigned& waiting, unsigned* s_flags) {
     if constexpr (W == 1) {
-        // one loop with one exit: here the warp stays together (one-word rounds are
-        // short; leaving one by one cost 20.5 ms against 14.3 on 1.6 G windows, and
-        // staying together cost two-word keys 1.74 ms against 1.39 on 0.19 G)
-        const unsigned lo = (unsigned)rec[0], khi = (unsigned)(rec[0] >> 32), klo = lo + 1u;
-        const unsigned hsh = (lo & ~63u) * 0x9E3779B1u + khi * 0x85EBCA77u;
-        unsigned g = __umulhi(hsh, ngroups), it = 0, sl = 0;
-        bool pending = have, hit = false;
-        while (pending) {
-            const unsigned ga = t.tail + 16 * g;
-            const uint4 a = lds128(ga);
-            const bool e0 = same_tail(a.x, a.y, klo, khi), e1 = same_tail(a.z, a.w, klo, khi);
-            hit = e0 || e1;
-            const bool full = !hit && a.z != 0u;
-            pending = full;
-            sl = 2 * g + (e1 ? 1u : 0u);
-            if (!hit && a.z == 0u) {
-                const unsigned occ = a.x ? 1u : 0u;
-                const unsigned long long old = claim64(ga + 8 * occ, rec[0] + 1ull);
-                if (old != 0ull) {  // taken: by this key, or by another (the group is read again)
-                    sl = 2 * g + occ;
-                    hit = same_tail((unsigned)old, (unsigned)(old >> 32), klo, khi);
-                    pending = !hit;
-                }
-            }
-            if (full) {
-                g += (hsh >> 8 & 255u) | 1u;
-                g -= g >= ngroups ? ngroups : 0u;
-                if (++it == kMaxRounds) {
-                    pending = false;
-                    atomicOr(s_flags, kLeafFull);
-                }
-            }
-        }
-        if (hit) {
-            const unsigned l = ext_left(lo), r = ext_right(lo);
-            bump(t, sl, l ? l - 1 : 4u);  // every counted window has exactly one left lane (the first: its code)
-            if (r) bump(t, sl, 4u + r);
-        }
-        __syncwarp();
+        const unsigned hsh = leaf_hash(rec[0]);
+        probe_round(t, rec[0], have, __umulhi(hsh, ngroups), 0u, hsh, ngroups, waiting, s_flags);
+        while (waiting >= 32u) probe_queue(t, ngroups, waiting, s_flags);
     } else {
         int slot = kClaimed;
         if (have) slot = find_slot<W>(t, rec, ngroups);
-        if (slot >= 0) {
-            const unsigned l = ext_left(rec[W - 1]), r = ext_right(rec[W - 1]);
-            bump(t, (unsigned)slot, l ? l - 1 : 4u);
-            if (r) bump(t, (unsigned)slot, 4u + r);
-        } else if (slot != kClaimed) {
-            atomicOr(s_flags, slot == kGaveUp ? kLeafTimeout : kLeafFull);
-        }
+        if (slot >= 0) tally(t, (unsigned)slot, rec[W - 1]);
+        else if (slot != kClaimed) atomicOr(s_flags, slot == kGaveUp ? kLeafTimeout : kLeafFull);
         __syncwarp();
     }
 }
 
-// Clears a warp's slice [s0, s0 + per) of the table (per a multiple of 32).
+// The records still waiting after a leaf's last one.
+template <int W>
+__device__ __forceinline__ void count_waiting(const Table& t, unsigned ngroups, unsigned& waiting, unsigned* s_flags) {
+    if constexpr (W == 1)
+        while (waiting) probe_queue(t, ngroups, waiting, s_flags);
+}
+
+// Clears a warp's slice [s0, s0 + per) of the table (per a multiple of 4).
 template <int W>
 __device__ __forceinline__ void clear_slice(const Table& t, unsigned s0, unsigned per) {
     const unsigned lane = threadIdx.x & 31;
@@ -339,7 +393,7 @@ __device__ __forceinline__ void clear_slice(const Table& t, unsigned s0, unsigne
     }
 }
 
-// Clears the whole table (all threads of the CTA; cap a multiple of 512).
+// Clears the whole table (all threads of the CTA; cap a multiple of 64).
 template <int W>
 __device__ __forceinline__ void clear_table(const Table& t, unsigned cap) {
     clear_slice<W>(t, (threadIdx.x >> 5) * (cap / kLeafWarps), cap / kLeafWarps);
@@ -356,10 +410,10 @@ __device__ __forceinline__ void sweep_table(const Job& j, const Table& t, const 
                                             unsigned& distinct) {
     const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned plane = 4 * t.stride;
-    const unsigned per = cap / kLeafWarps;  // a multiple of 32
+    const unsigned per = cap / kLeafWarps;  // a multiple of 4
     const unsigned s0 = wid * per;
     const unsigned more = j.min_count - 1;  // records besides the one that claimed the slot
-    const unsigned mylist = t.list + 4 * s0, before = (1u << lane) - 1u;
+    const unsigned mylist = t.list + 2 * s0, before = (1u << lane) - 1u;
     unsigned count = 0;
     for (unsigned b = 0; b < per; b += 128) {
         unsigned occ[4], p0[4], p1[4], p2[4];
@@ -399,7 +453,7 @@ __device__ __forceinline__ void sweep_table(const Job& j, const Table& t, const 
             distinct += occ[q] != 0u ? 1u : 0u;
             const unsigned m = __ballot_sync(0xffffffffu, ok);
             if (ok)
-                sts32(mylist + 4 * (count + __popc(m & before)), s0 + (W == 2 ? b + 32 * q + lane : b + 4 * lane + q));
+                sts16(mylist + 2 * (count + __popc(m & before)), s0 + (W == 2 ? b + 32 * q + lane : b + 4 * lane + q));
             count += __popc(m);
         }
     }
@@ -408,7 +462,7 @@ __device__ __forceinline__ void sweep_table(const Job& j, const Table& t, const 
     if (lane == 0 && count) wbase = atomicAdd(j.out_n, (unsigned long long)count);
     wbase = __shfl_sync(0xffffffffu, wbase, 0);
     for (unsigned i = lane; i < count; i += 32) {
-        const unsigned s = lds32(mylist + 4 * i);
+        const unsigned s = lds16(mylist + 2 * i);
         const unsigned long long pos = wbase + i;
         const unsigned long long tl = slot_tail<W>(t, s);
         unsigned pl[kLanePlanes];
@@ -465,7 +519,7 @@ __device__ __forceinline__ unsigned count_in_ranges(const Job& j, const Table& t
     unsigned rb = 0, rs = 0;
     for (;;) {
         const unsigned shift = free_bits - rb, rmask = (1u << rb) - 1u;
-        unsigned rwin = 0;
+        unsigned rwin = 0, waiting = 0;
         for (unsigned i0 = 0; i0 < n; i0 += kLeafThreads) {
             const unsigned i = i0 + threadIdx.x;
             unsigned long long rec[W];
@@ -473,8 +527,9 @@ __device__ __forceinline__ unsigned count_in_ranges(const Job& j, const Table& t
             for (int w = 0; w < W; ++w) rec[w] = i < n ? src[(size_t)i * W + w] : 0ull;
             const bool in = i < n && ((unsigned)((rec[W - 1] >> 6) >> shift) & rmask) == rs;
             rwin += in ? 1u : 0u;
-            count_record<W>(t, rec, in && !*(volatile unsigned*)s_flags, groups_of<W>(cap), s_flags);
+            count_record<W>(t, rec, in && !*(volatile unsigned*)s_flags, groups_of<W>(cap), waiting, s_flags);
         }
+        count_waiting<W>(t, groups_of<W>(cap), waiting, s_flags);
         __syncthreads();
         const unsigned flags = *(volatile unsigned*)s_flags;
         if (flags == kLeafFull && rb < max_rb) {  // split the range in two
@@ -532,6 +587,7 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_split_kernel(const Job* 
     t.heads = t.tail + 8 * cap_max;
     t.lanes = t.heads + 8 * (W - 1) * cap_max;
     t.list = t.lanes + 4 * kLanePlanes * cap_max;
+    t.queue = t.list + 2 * cap_max + (threadIdx.x >> 5) * kQueue * 12;  // 128-byte aligned
     bool init = false;
     for (unsigned ji = 0; ji < n_jobs; ++ji) {
         const Job& j = jobs[ji];
@@ -585,6 +641,7 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_kernel(const Job* __rest
     t.heads = t.tail + 8 * cap_max;
     t.lanes = t.heads + 8 * (W - 1) * cap_max;
     t.list = t.lanes + 4 * kLanePlanes * cap_max;
+    t.queue = t.list + 2 * cap_max + (threadIdx.x >> 5) * kQueue * 12;  // 128-byte aligned
     clear_table<W>(t, cap_max);
     if (threadIdx.x == 0) s_flags = 0;
 
@@ -650,8 +707,11 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_kernel(const Job* __rest
         }
         // ---------------------------------------------------------- count
         const unsigned n = (unsigned)li.n;  // below 65 536, as is the ratio (at most 65 536)
-        const unsigned want = (unsigned)(((unsigned long long)n * j.table_ratio_num) >> 16) + 512u;
-        const unsigned cap = want < cap_max ? ((want + 511u) & ~511u) : cap_max;
+        // twice the expected keys and 1024: emptier tables probe less than their
+        // sweep costs (256 / 512 / 1280 in place of 1024 at k = 55 with the gate:
+        // 1.57 / 1.45 / 1.28 ms)
+        const unsigned want = (unsigned)(((unsigned long long)n * j.table_ratio_num) >> 16) + 1024u;
+        const unsigned cap = want < cap_max ? ((want + 63u) & ~63u) : cap_max;
         const unsigned ngroups = groups_of<W>(cap);
         if (threadIdx.x == kLeafThreads - 1) {
             LeafInfo x;
@@ -659,14 +719,16 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_kernel(const Job* __rest
             if (ng < total) x = leaf_info(jobs[nji], nleaf);
             s_next = x;
         }
+        unsigned waiting = 0;  // records in this warp's queue
         for (unsigned first = 0; first < n; first += B) {
             if (first) load_batch<W>(li, first, batch);
-            if (*(volatile unsigned*)&s_flags) break;
+            if (__any_sync(0xffffffffu, *(volatile unsigned*)&s_flags != 0u)) break;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                count_record<W>(t, batch[u], first + u * kLeafThreads + threadIdx.x < n, ngroups, &s_flags);
+                count_record<W>(t, batch[u], first + u * kLeafThreads + threadIdx.x < n, ngroups, waiting, &s_flags);
             }
         }
+        count_waiting<W>(t, ngroups, waiting, &s_flags);
         __syncthreads();
         const unsigned flags = s_flags;
         // the next leaf's first batch loads while this one is swept
