@@ -153,9 +153,9 @@ struct Job {
     unsigned int* fb_list;
     unsigned int* fb_n;
     unsigned int fb_cap;
-    // Bloom gate (gate.cu): F2, 2^gate_bits words; null = every window is emitted
+    // Bloom gate (gate.cu): F2, gate_words words; null = every window is emitted
     const unsigned long long* gate;
-    unsigned gate_bits;
+    unsigned long long gate_words;
     // classification
     unsigned min_count, ext_mode, t_base, err_num, err_den, t_ext;
     // sizing: level-2 leaf capacity = mean * l2_slack_num / 256 + 256 records;

@@ -14,7 +14,9 @@
 // (count 1) and dropped by the count filter.
 //
 // Filters are blocked: a key touches one 64-bit word of each, setting four
-// bits, with one atomicOr per filter.
+// bits, with one atomicOr per filter.  Bound by the random 8-byte atomics
+// (32-byte sectors read and written back where the L2 misses): a filter has
+// exactly the words it was sized for.
 #include "kernels.h"
 #include "roll.cuh"
 
@@ -22,7 +24,7 @@ namespace kmer {
 
 template <int W, bool HI>
 __global__ void __launch_bounds__(256) gate_kernel(const Job j, unsigned long long* __restrict__ f1,
-                                                   unsigned long long* __restrict__ f2, const unsigned log2_words,
+                                                   unsigned long long* __restrict__ f2, const unsigned long long words,
                                                    unsigned long long* __restrict__ counts) {
     const unsigned long long r = blockIdx.x * 256ull + threadIdx.x;
     unsigned windows = 0, first = 0, second = 0;
@@ -34,7 +36,7 @@ __global__ void __launch_bounds__(256) gate_kernel(const Job j, unsigned long lo
             unsigned lc, rc;
             if (!roll.step(t, key, lc, rc)) continue;
             ++windows;
-            const GateProbe p = gate_probe(gate_hash<W>(key), log2_words);
+            const GateProbe p = gate_probe(gate_hash<W>(key), words);
             const unsigned long long o1 = atomicOr(f1 + p.word, p.mask);
             if ((o1 & p.mask) != p.mask) {
                 ++first;  // first sighting (or a false positive of F1)
@@ -58,24 +60,24 @@ __global__ void __launch_bounds__(256) gate_kernel(const Job j, unsigned long lo
 }
 
 template <int W, bool HI>
-static cudaError_t launch_gate_w(const Job& j, unsigned long long* f1, unsigned long long* f2, unsigned log2_words,
+static cudaError_t launch_gate_w(const Job& j, unsigned long long* f1, unsigned long long* f2, unsigned long long words,
                                  unsigned long long* counts, cudaStream_t s) {
     if (j.n_reads == 0) return cudaSuccess;
     const unsigned long long grid = (j.n_reads + 255) / 256;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidValue;
-    gate_kernel<W, HI><<<(unsigned)grid, 256, 0, s>>>(j, f1, f2, log2_words, counts);
+    gate_kernel<W, HI><<<(unsigned)grid, 256, 0, s>>>(j, f1, f2, words, counts);
     return cudaGetLastError();
 }
 
-cudaError_t launch_gate(const Job& j, unsigned long long* f1, unsigned long long* f2, unsigned log2_words,
+cudaError_t launch_gate(const Job& j, unsigned long long* f1, unsigned long long* f2, unsigned long long words,
                         unsigned long long* counts, cudaStream_t s) {
     switch (j.g.W) {
         case 1:
-            return j.g.k >= 17 ? launch_gate_w<1, true>(j, f1, f2, log2_words, counts, s)
-                               : launch_gate_w<1, false>(j, f1, f2, log2_words, counts, s);
-        case 2: return launch_gate_w<2, false>(j, f1, f2, log2_words, counts, s);
-        case 3: return launch_gate_w<3, false>(j, f1, f2, log2_words, counts, s);
-        case 4: return launch_gate_w<4, false>(j, f1, f2, log2_words, counts, s);
+            return j.g.k >= 17 ? launch_gate_w<1, true>(j, f1, f2, words, counts, s)
+                               : launch_gate_w<1, false>(j, f1, f2, words, counts, s);
+        case 2: return launch_gate_w<2, false>(j, f1, f2, words, counts, s);
+        case 3: return launch_gate_w<3, false>(j, f1, f2, words, counts, s);
+        case 4: return launch_gate_w<4, false>(j, f1, f2, words, counts, s);
     }
     return cudaErrorInvalidValue;
 }

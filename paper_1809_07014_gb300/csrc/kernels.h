@@ -62,9 +62,9 @@ cudaError_t launch_index_build(unsigned W, const unsigned long long* keys, unsig
                                unsigned* idx, unsigned long long cap, int num_sms, cudaStream_t s);
 
 // Bloom gate (gate.cu): adds every window's key of the job's reads to filter
-// f1, and keys already in f1 to f2 (both 2^log2_words words, zeroed by the
+// f1, and keys already in f1 to f2 (both `words` words, zeroed by the
 // caller); counts[0..2] += windows, first sightings, keys entering f2.
-cudaError_t launch_gate(const Job& j, unsigned long long* f1, unsigned long long* f2, unsigned log2_words,
+cudaError_t launch_gate(const Job& j, unsigned long long* f1, unsigned long long* f2, unsigned long long words,
                         unsigned long long* counts, cudaStream_t s);
 
 // Merge (Algorithm 1): k-mers of a second canonical, distinct set (bkeys,

@@ -226,23 +226,23 @@ __device__ __forceinline__ unsigned long long gate_hash(const unsigned long long
     return h;
 }
 
-// The filter word (top log2_words bits of the hash) and four bits within it
-// (four 6-bit fields of the low bits).
+// The filter word (the hash's share of `words`, from its top bits) and four
+// bits within it (four 6-bit fields of the low bits).
 struct GateProbe {
     unsigned long long word, mask;
 };
-__device__ __forceinline__ GateProbe gate_probe(unsigned long long h, unsigned log2_words) {
+__device__ __forceinline__ GateProbe gate_probe(unsigned long long h, unsigned long long words) {
     GateProbe p;
-    p.word = log2_words ? h >> (64 - log2_words) : 0ull;
+    p.word = __umul64hi(h, words);
     p.mask = (1ull << (h & 63)) | (1ull << ((h >> 6) & 63)) | (1ull << ((h >> 12) & 63)) | (1ull << ((h >> 18) & 63));
     return p;
 }
 
 // The key is in the gate's filter (every bit of its probe set).
 template <int W>
-__device__ __forceinline__ bool gate_has(const unsigned long long* f, unsigned log2_words,
+__device__ __forceinline__ bool gate_has(const unsigned long long* f, unsigned long long words,
                                          const unsigned long long (&key)[W]) {
-    const GateProbe p = gate_probe(gate_hash<W>(key), log2_words);
+    const GateProbe p = gate_probe(gate_hash<W>(key), words);
     return (__ldg(f + p.word) & p.mask) == p.mask;
 }
 

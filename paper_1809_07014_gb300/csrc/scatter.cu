@@ -72,7 +72,7 @@ __device__ __forceinline__ void scatter_tile(const Job& j, const unsigned long l
     L1Dest dest{j.l1_fill, j.l1_start, j.l1_cap};
     const unsigned pass = j.pass;
     const unsigned long long* gate = j.gate;  // Bloom gate (GATE): emit only keys in F2
-    const unsigned gate_bits = j.gate_bits;
+    const unsigned long long gate_words = j.gate_words;
     unsigned emitted = 0;
     for (unsigned s0 = 0; s0 < steps; s0 += R) {
         unsigned m[R];
@@ -83,7 +83,7 @@ __device__ __forceinline__ void scatter_tile(const Job& j, const unsigned long l
             if (t < end) {
                 unsigned long long key[W], rec[W];
                 unsigned lc = 0, rc = 0, bucket = 0;
-                if (roll.step(t++, key, lc, rc) && (!GATE || gate_has<W>(gate, gate_bits, key)) &&
+                if (roll.step(t++, key, lc, rc) && (!GATE || gate_has<W>(gate, gate_words, key)) &&
                     make_record<W>(g, pass, key, lc, rc, rec, bucket)) {
                     m[s] = (bucket << 16) | atomicAdd(&b.hist[bucket], 1u);
                     if constexpr (W == 2 || W == 4) {
