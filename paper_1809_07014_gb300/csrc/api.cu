@@ -172,7 +172,8 @@ struct kmer_analysis {
     std::vector<const kmer_readset*> submitted;
     std::vector<kmer_readset*> owned;
     // device buffers
-    DevBuf l1_rec, l1_start, l1_cap, l1_fill;
+    DevBuf l1_rec;
+    DevBuf d_desc;  // level-1 starts, capacities and fills, work maps and job descriptors of a pass
     DevBuf l2_rec, l2_base, l2_leafcap, l2_fill, l2_leaf_start, tile_prefix;
     DevBuf out_keys, out_count, out_ext, out_cls;
     DevBuf fb_list, split_list, hbm, misc;
@@ -192,7 +193,7 @@ struct kmer_analysis {
     unsigned long long lk_cap = 0;     // index slots; 0 = no index for the current results
     bool lk_streamed = false;          // the current results answered a lookup without an index
     DevBuf lk_wanted;                  // scratch of such a lookup
-    DevBuf d_ajob, d_sjobs, d_tile_off, d_leaf_off, d_job_tile_off;  // job descriptors and work maps
+    DevBuf d_ajob, d_leaf_off, d_job_tile_off;  // descriptor and work maps of a wave or a retry
     unsigned long long out_cap = 0, fb_cap = 0;
     Misc* host_misc = nullptr;  // pinned
     // profiling (KMER_FLAG_PROFILE): one begin/end event pair per stage
@@ -220,15 +221,17 @@ struct kmer_analysis {
     double l1_imbalance = 0.0;
     std::vector<unsigned long long> l1_prev_fill;
     unsigned long long l1_prev_windows = 0;
+    // device memory found free by the last query that asked, and its windows
+    size_t plan_budget = 0;
+    unsigned long long plan_windows = 0;
     kmer_analysis_stats st{};
 
     unsigned W() const { return (2 * p.k + 63) / 64; }
     size_t device_bytes() const {
-        const DevBuf* bs[] = {&l1_rec, &l1_start, &l1_cap, &l1_fill, &l2_rec, &l2_base, &l2_leafcap, &l2_fill,
+        const DevBuf* bs[] = {&l1_rec, &d_desc, &l2_rec, &l2_base, &l2_leafcap, &l2_fill,
                               &l2_leaf_start, &tile_prefix, &out_keys, &out_count, &out_ext, &out_cls,
                               &fb_list, &split_list, &hbm, &misc, &lk_index, &lk_keys, &lk_out, &lk_wanted, &d_ajob,
-                              &d_sjobs, &d_tile_off, &d_leaf_off,
-                              &d_job_tile_off, &gate1, &gate2, &gate_cnt, &trav_scratch, &trav_bases, &trav_off,
+                              &d_leaf_off, &d_job_tile_off, &gate1, &gate2, &gate_cnt, &trav_scratch, &trav_bases, &trav_off,
                               &trav_tot, &sort_buf};
         size_t t = 0;
         for (auto* b : bs) t += b->bytes;
@@ -351,11 +354,10 @@ int pack_readset(kmer_readset* rs, const char* bases, const uint8_t* quals, cons
     CK(launch_read_geometry(d_off, n_reads, rs->nblk.as<unsigned long long>(), st, bad, s));
     CK(exclusive_scan_u64(rs->nblk.as<unsigned long long>(), rs->blk_off.as<unsigned long long>(), n_reads,
                           rs->scratch.p, s));
-    // gather the totals next to the histogram so that one copy brings everything back
+    // the total next to the histogram (and the offsets' ends, which the geometry
+    // kernel left there), so that one copy brings everything back
     CK(cudaMemcpyAsync(st + kLenHist + 2, rs->blk_off.as<unsigned long long>() + n_reads, 8,
                        cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(st + kLenHist + 3, d_off, 8, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(st + kLenHist + 4, d_off + n_reads, 8, cudaMemcpyDeviceToDevice, s));
     std::vector<unsigned long long> host(kLenHist + 5);
     CK(cudaMemcpyAsync(host.data(), st, host.size() * 8, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -653,21 +655,17 @@ struct WaveTotals {
     unsigned long long out_n = 0, windows = 0, distinct = 0, splits = 0, emitted = 0;
 };
 
-// Level-2 stages (repartition, leaves, fallbacks) of one pass over the
-// level-1 buckets [b0, b0 + nb) (a wave, or all of them), with their retries.
-// `fresh`: reset the device counters first (keeping out_n and the scatter's
-// emitted count).  Sets *rescatter when a level-1 bucket overflowed.
-int run_level2(kmer_analysis* h, Job j, unsigned b0, unsigned nb, unsigned long long l2_capacity, unsigned cap_max,
-               bool fresh, WaveTotals& tot, bool* rescatter) {
+// Descriptor of the level-2 stages over the level-1 buckets [b0, b0 + nb), its
+// buffers made large enough.
+int level2_job(kmer_analysis* h, Job& j, unsigned b0, unsigned nb, unsigned long long l2_capacity) {
     const Geometry g = j.g;
-    const unsigned P1 = 1u << g.p1, P2 = 1u << g.p2, W = g.W;
+    const unsigned P1 = 1u << g.p1, W = g.W;
     const unsigned Pw = g.p2 ? nb << g.p2 : nb;  // leaves of the wave
     j.bucket0 = b0;
     j.n_buckets = (b0 == 0 && nb == P1) ? 0 : nb;
     j.l1_start += b0;
     j.l1_cap += b0;
     j.l1_fill += b0;
-    std::vector<unsigned long long> exact_leaf;  // exact level-2 layout after an overflow
     if (g.p2) {
         TRY(h->l2_rec.fit(l2_capacity * 8 * W + 64));
         TRY(h->l2_base.ensure(nb * 8ull));
@@ -683,27 +681,49 @@ int run_level2(kmer_analysis* h, Job j, unsigned b0, unsigned nb, unsigned long 
     }
     TRY(h->split_list.ensure((size_t)Pw * 4));  // every leaf could need key ranges
     fill_job_outputs(h, j);
+    j.l2_capacity = l2_capacity;
+    return KMER_OK;
+}
+
+// Level-2 stages (repartition, leaves, fallbacks) of one pass over the
+// level-1 buckets [b0, b0 + nb) (a wave, or all of them), with their retries.
+// `fresh`: reset the device counters first (keeping out_n and the scatter's
+// emitted count).  d_first / d_leaf: the first attempt's descriptor and leaf
+// map if they are on the device already.  Sets *rescatter when a level-1
+// bucket overflowed.
+int run_level2(kmer_analysis* h, Job j, unsigned b0, unsigned nb, unsigned long long l2_capacity, unsigned cap_max,
+               bool fresh, WaveTotals& tot, bool* rescatter, const Job* d_first, const unsigned long long* d_leaf) {
+    const Geometry g = j.g;
+    const unsigned W = g.W;
+    const unsigned Pw = g.p2 ? nb << g.p2 : nb;  // leaves of the wave
+    std::vector<unsigned long long> exact_leaf;  // exact level-2 layout after an overflow
+    TRY(level2_job(h, j, b0, nb, l2_capacity));
     if (fresh) TRY(reset_misc(h, tot.out_n, tot.emitted));
-    const std::vector<unsigned long long> leaf_off = {0ull, (unsigned long long)Pw};
-    TRY(upload(h, h->d_leaf_off, leaf_off));
+    if (!d_leaf) {
+        TRY(upload(h, h->d_leaf_off, std::vector<unsigned long long>{0ull, (unsigned long long)Pw}));
+        d_leaf = h->d_leaf_off.as<unsigned long long>();
+    }
     TRY(h->d_job_tile_off.ensure(2 * 8));
     for (unsigned sub_attempt = 0;; ++sub_attempt) {
         if (sub_attempt > 8) return fail(KMER_ERR_TABLE_FULL, "leaf buffers still too small after retries");
         j.l2_capacity = exact_leaf.empty() ? l2_capacity : ~0ull;
-        TRY(upload(h, h->d_ajob, std::vector<Job>{j}));
+        const Job* dj = sub_attempt == 0 ? d_first : nullptr;
+        if (!dj) {
+            TRY(upload(h, h->d_ajob, std::vector<Job>{j}));
+            dj = h->d_ajob.as<Job>();
+        }
         if (g.p2) {
             CK(cudaMemsetAsync(h->l2_fill.p, 0, Pw * 8ull, h->stream));
             TRY(prof_begin(h, kmer_analysis::STG_REPART));
-            CK(launch_l2_plan(h->d_ajob.as<Job>(), 1, h->d_job_tile_off.as<unsigned long long>(), h->stream));
-            CK(launch_repart(W, h->d_ajob.as<Job>(), h->d_job_tile_off.as<unsigned long long>(), 1, g.p2,
+            CK(launch_l2_plan(dj, 1, h->d_job_tile_off.as<unsigned long long>(), h->stream));
+            CK(launch_repart(W, dj, h->d_job_tile_off.as<unsigned long long>(), 1, g.p2,
                              h->num_sms, h->stream));
             TRY(prof_end(h, kmer_analysis::STG_REPART));
             h->st.launches += 3;
         }
         TRY(prof_begin(h, kmer_analysis::STG_LEAF));
-        CK(launch_leaf(W, h->d_ajob.as<Job>(), h->d_leaf_off.as<unsigned long long>(), 1, Pw, cap_max, h->num_sms,
-                       h->stream));
-        CK(launch_leaf_split(W, h->d_ajob.as<Job>(), 1, cap_max, h->num_sms, h->stream));
+        CK(launch_leaf(W, dj, d_leaf, 1, Pw, cap_max, h->num_sms, h->stream));
+        CK(launch_leaf_split(W, dj, 1, cap_max, h->num_sms, h->stream));
         TRY(prof_end(h, kmer_analysis::STG_LEAF));
         h->st.launches += 2;
         TRY(read_misc(h));
@@ -799,12 +819,6 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
         // the repartition's bulk copies start on 16-byte boundaries of this region
         if (reinterpret_cast<uintptr_t>(h->l1_rec.p) & 15)
             return fail(KMER_ERR_CUDA, "level-1 record buffer is not 16-byte aligned");
-        TRY(h->l1_start.ensure((P1 + 1) * 8));
-        TRY(h->l1_cap.ensure(P1 * 8));
-        TRY(h->l1_fill.ensure(P1 * 8));
-        CK(cudaMemcpyAsync(h->l1_start.p, starts.data(), (P1 + 1) * 8, cudaMemcpyHostToDevice, h->stream));
-        CK(cudaMemcpyAsync(h->l1_cap.p, caps.data(), P1 * 8, cudaMemcpyHostToDevice, h->stream));
-        CK(cudaMemsetAsync(h->l1_fill.p, 0, P1 * 8, h->stream));
         // level-2 records of all buckets: sum over buckets of P2 leaves of
         // (mean * slack + 256) records, mean <= n_b / P2 + 1
         const unsigned long long l2_full =
@@ -818,14 +832,38 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
             TRY(h->fb_list.ensure(64 * 4));
             h->fb_cap = 64;
         }
+        // every table of the pass lies in one buffer and goes up in one copy
+        // (seven copies cost about 35 us of host time, during which the GPU idles)
+        size_t n_sets = 0;
+        unsigned long long all_reads = 0;
+        for (const kmer_readset* rs : h->submitted) {
+            n_sets += rs->n_reads != 0;
+            all_reads += rs->n_reads;
+        }
+        const unsigned seg_bits = scatter_seg_bits(all_reads, h->num_sms), tile_reads = scatter_tile_reads(seg_bits);
+        size_t bytes = 0;
+        auto place = [&](size_t n) {
+            const size_t at = bytes;
+            bytes += (n + 255) & ~size_t(255);
+            return at;
+        };
+        const size_t at_start = place((P1 + 1) * 8), at_cap = place(P1 * 8), at_fill = place(P1 * 8);
+        const size_t at_tiles = place((n_sets + 1) * 8), at_leaf = place(2 * 8);
+        const size_t at_sjobs = place(n_sets * sizeof(Job)), at_ajob = place(sizeof(Job));
+        TRY(h->d_desc.ensure(bytes));
+        char* const desc = h->d_desc.as<char>();
+        unsigned long long* const l1_fill = reinterpret_cast<unsigned long long*>(desc + at_fill);
+        std::vector<char> host(bytes, 0);  // the fills start at zero
+        std::memcpy(host.data() + at_start, starts.data(), (P1 + 1) * 8);
+        std::memcpy(host.data() + at_cap, caps.data(), P1 * 8);
         TRY(reset_misc(h, out_start));
         Job j{};
         j.g = g;
         j.pass = pass;
         j.l1_rec = h->l1_rec.as<unsigned long long>();
-        j.l1_start = h->l1_start.as<unsigned long long>();
-        j.l1_cap = h->l1_cap.as<unsigned long long>();
-        j.l1_fill = h->l1_fill.as<unsigned long long>();
+        j.l1_start = reinterpret_cast<unsigned long long*>(desc + at_start);
+        j.l1_cap = reinterpret_cast<unsigned long long*>(desc + at_cap);
+        j.l1_fill = l1_fill;
         fill_job_outputs(h, j);
         j.l2_slack_num = h->l2_slack_num;
         if (h->p.flags & KMER_FLAG_BLOOM_GATE) {
@@ -833,24 +871,30 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
             j.gate_words = h->gate_words;
         }
         // one scatter job per submitted readset, one CTA per tile of reads
-        unsigned long long all_reads = 0;
-        for (const kmer_readset* rs : h->submitted) all_reads += rs->n_reads;
-        const unsigned seg_bits = scatter_seg_bits(all_reads, h->num_sms), tile_reads = scatter_tile_reads(seg_bits);
-        std::vector<Job> sjobs;
-        std::vector<unsigned long long> tile_off(1, 0);
+        Job* const sjobs = reinterpret_cast<Job*>(host.data() + at_sjobs);
+        unsigned long long* const tile_off = reinterpret_cast<unsigned long long*>(host.data() + at_tiles);
+        size_t si = 0;
         for (const kmer_readset* rs : h->submitted) {
             if (rs->n_reads == 0) continue;
             Job js = j;
             set_readset(js, rs);
-            sjobs.push_back(js);
-            tile_off.push_back(tile_off.back() + (rs->n_reads + tile_reads - 1) / tile_reads);
+            std::memcpy(sjobs + si, &js, sizeof js);
+            tile_off[si + 1] = tile_off[si] + (rs->n_reads + tile_reads - 1) / tile_reads;
+            ++si;
         }
-        TRY(upload(h, h->d_sjobs, sjobs));
-        TRY(upload(h, h->d_tile_off, tile_off));
+        const unsigned long long tiles = tile_off[n_sets];
+        if (!waves) {  // the level-2 stages' first attempt
+            Job ja = j;
+            TRY(level2_job(h, ja, 0, P1, l2_full));
+            std::memcpy(host.data() + at_ajob, &ja, sizeof ja);
+            reinterpret_cast<unsigned long long*>(host.data() + at_leaf)[1] = (unsigned long long)P1 << g.p2;
+        }
+        CK(cudaMemcpyAsync(desc, host.data(), bytes, cudaMemcpyHostToDevice, h->stream));
         TRY(prof_begin(h, kmer_analysis::STG_SCATTER));
-        if (!sjobs.empty()) {
-            CK(launch_scatter(W, h->d_sjobs.as<Job>(), h->d_tile_off.as<unsigned long long>(), (unsigned)sjobs.size(),
-                              tile_off.back(), seg_bits, g.p1, g.k, j.gate != nullptr, h->stream));
+        if (n_sets) {
+            CK(launch_scatter(W, reinterpret_cast<Job*>(desc + at_sjobs),
+                              reinterpret_cast<unsigned long long*>(desc + at_tiles), (unsigned)n_sets, tiles, seg_bits,
+                              g.p1, g.k, j.gate != nullptr, h->stream));
             h->st.launches++;
         }
         TRY(prof_end(h, kmer_analysis::STG_SCATTER));
@@ -863,7 +907,7 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
             TRY(read_misc(h));
             if (h->host_misc->status & ST_L1_OVERFLOW) {
                 std::vector<unsigned long long> fill(P1);
-                CK(cudaMemcpyAsync(fill.data(), h->l1_fill.p, P1 * 8, cudaMemcpyDeviceToHost, h->stream));
+                CK(cudaMemcpyAsync(fill.data(), l1_fill, P1 * 8, cudaMemcpyDeviceToHost, h->stream));
                 CK(cudaStreamSynchronize(h->stream));
                 for (unsigned b = 0; b < P1; ++b) caps[b] = std::max(caps[b], fill[b]);
                 h->st.retries++;
@@ -871,7 +915,7 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
             }
             tot.emitted = h->host_misc->stats[2];
             std::vector<unsigned long long> fill(P1);
-            CK(cudaMemcpyAsync(fill.data(), h->l1_fill.p, P1 * 8, cudaMemcpyDeviceToHost, h->stream));
+            CK(cudaMemcpyAsync(fill.data(), l1_fill, P1 * 8, cudaMemcpyDeviceToHost, h->stream));
             CK(cudaStreamSynchronize(h->stream));
             const unsigned long long room = std::max<unsigned long long>(avail / (8ull * W), 1);
             wave_start.assign(1, 0);
@@ -894,10 +938,11 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
         bool rescatter = false;
         for (size_t w = 0; w + 1 < wave_start.size() && !rescatter; ++w)
             TRY(run_level2(h, j, wave_start[w], wave_start[w + 1] - wave_start[w], l2_cap, cap_max, waves, tot,
-                           &rescatter));
+                           &rescatter, waves ? nullptr : reinterpret_cast<Job*>(desc + at_ajob),
+                           waves ? nullptr : reinterpret_cast<unsigned long long*>(desc + at_leaf)));
         if (rescatter) {  // level-1 overflow: take the exact bucket demand and re-scatter
             std::vector<unsigned long long> fill(P1);
-            CK(cudaMemcpyAsync(fill.data(), h->l1_fill.p, P1 * 8, cudaMemcpyDeviceToHost, h->stream));
+            CK(cudaMemcpyAsync(fill.data(), l1_fill, P1 * 8, cudaMemcpyDeviceToHost, h->stream));
             CK(cudaStreamSynchronize(h->stream));
             for (unsigned b = 0; b < P1; ++b) caps[b] = std::max(caps[b], fill[b]);
             h->st.retries++;
@@ -907,7 +952,7 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
             return fail(KMER_ERR_CUDA, "internal: %llu windows emitted but %llu counted", tot.emitted, tot.windows);
         if (pass_windows >= (1ull << 26)) {  // learn the buckets' imbalance for the next large query
             std::vector<unsigned long long> fill(P1);
-            CK(cudaMemcpyAsync(fill.data(), h->l1_fill.p, P1 * 8, cudaMemcpyDeviceToHost, h->stream));
+            CK(cudaMemcpyAsync(fill.data(), l1_fill, P1 * 8, cudaMemcpyDeviceToHost, h->stream));
             CK(cudaStreamSynchronize(h->stream));
             const double em = (double)tot.emitted / (double)P1;
             if (em > 0) {
@@ -1084,7 +1129,15 @@ int do_query(kmer_analysis* h) {
             const unsigned W = h->W();
             const unsigned cap_max = leaf_table_cap(W, h->leaf_smem_budget);
             size_t budget = h->p.memory_budget;
-            if (!budget) budget = (size_t)(0.85 * (double)(free_device_bytes() + h->device_bytes()));
+            if (!budget) {
+                // asking for the free memory takes the driver 26 us: a query of about the
+                // last one's size (whose buffers are still here) plans with the last answer
+                if (!h->plan_budget || windows > h->plan_windows || windows < h->plan_windows - h->plan_windows / 8) {
+                    h->plan_budget = (size_t)(0.85 * (double)(free_device_bytes() + h->device_bytes()));
+                    h->plan_windows = windows;
+                }
+                budget = h->plan_budget;
+            }
             // output sized from the previous query or a fraction of the windows, at most
             // 35 % of the budget on a first query; grown on demand
             const unsigned long long out_bytes_per = 8ull * W + 4 + 32 + 2;
@@ -1301,6 +1354,7 @@ int kmer_analysis_query(kmer_analysis_t* h, kmer_result_view* out) {
     int rc = do_query(h);
     if (rc != KMER_OK) {
         h->have_result = false;
+        h->plan_budget = 0;
         cudaGetLastError();
         return rc;
     }
@@ -1330,6 +1384,7 @@ int kmer_analysis_query_into(kmer_analysis_t* h, uint64_t* keys, uint32_t* count
         const int rc = do_query(h);
         if (rc != KMER_OK) {
             h->have_result = false;
+            h->plan_budget = 0;
             cudaGetLastError();
             return rc;
         }
@@ -1377,6 +1432,7 @@ int kmer_analysis_query_into(kmer_analysis_t* h, uint64_t* keys, uint32_t* count
     h->out_cap = own_cap;
     if (rc != KMER_OK) {
         h->have_result = false;
+        h->plan_budget = 0;
         cudaGetLastError();
         return rc;
     }
@@ -1684,7 +1740,7 @@ int kmer_analysis_destroy(kmer_analysis_t* h) {
     if (h->stream) cudaStreamSynchronize(h->stream);
     else cudaDeviceSynchronize();
     kmer_analysis_reset(h);
-    DevBuf* bs[] = {&h->l1_rec, &h->l1_start, &h->l1_cap, &h->l1_fill, &h->l2_rec, &h->l2_base, &h->l2_leafcap,
+    DevBuf* bs[] = {&h->l1_rec, &h->d_desc, &h->l2_rec, &h->l2_base, &h->l2_leafcap,
                     &h->l2_fill, &h->l2_leaf_start, &h->tile_prefix, &h->out_keys, &h->out_count, &h->out_ext,
                     &h->out_cls, &h->fb_list, &h->split_list, &h->hbm, &h->misc, &h->lk_index, &h->lk_keys,
                     &h->lk_out};

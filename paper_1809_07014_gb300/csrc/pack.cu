@@ -105,6 +105,10 @@ __global__ void __launch_bounds__(256) read_geometry_kernel(const unsigned long 
                                                             unsigned long long* nblk, unsigned long long* len_stats,
                                                             unsigned int* bad) {
     __shared__ unsigned long long hist[kLenHist];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {  // after the histogram, the flags and the blocks' total
+        len_stats[kLenHist + 3] = offsets[0];
+        len_stats[kLenHist + 4] = offsets[n];
+    }
     for (int i = threadIdx.x; i < kLenHist; i += blockDim.x) hist[i] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
