@@ -142,7 +142,10 @@ Geometry plan_geometry(unsigned k, unsigned long long windows, unsigned long lon
     }
     const unsigned lb = p - ps;
     unsigned p1, p2;
-    if (lb <= 11) {
+    // one level up to 2^10 leaves: a flush of 4096 records into 2^11 destinations
+    // makes a reservation for every other record (4 Mbases at k = 21: 405 us in
+    // one level, 354 in two; at 2^10 one level is the faster by 3 to 10 %)
+    if (lb <= 10) {
         p1 = lb;
         p2 = 0;
     } else {
