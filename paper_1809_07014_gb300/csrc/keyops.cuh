@@ -46,12 +46,6 @@ __device__ __forceinline__ unsigned get_base(const unsigned long long (&key)[W],
     return (unsigned)(key[W - 1 - pos / 64] >> (pos % 64)) & 3u;
 }
 
-template <int W>
-__device__ __forceinline__ void set_base(unsigned long long (&key)[W], unsigned k, unsigned i, unsigned b) {
-    const unsigned pos = 2 * (k - 1 - i);
-    key[W - 1 - pos / 64] |= (unsigned long long)b << (pos % 64);
-}
-
 // Position of `key` among the survivors through the index, or kIdxEmpty.
 template <int W>
 __device__ __forceinline__ unsigned index_find(const unsigned long long (&key)[W], unsigned k,
