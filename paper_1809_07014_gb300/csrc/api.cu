@@ -1580,13 +1580,15 @@ int kmer_analysis_merge_contigs(kmer_analysis_t* h, const char* contigs, const u
         // anywhere in the contigs, DEAD_END when none, FORK when several
         // A contig longer than kMergePiece bases is cut into pieces of that
         // many bases overlapping by k + 1, since one thread rolls the windows of
-        // one read and contigs can be millions of bases long (pieces of 16 k
-        // bases, at least 1024: the overlaps cost at most a sixteenth more
-        // windows, and the pieces keep the GPU's threads busy).  Each window and
-        // both its extension bases then lie whole in some piece; a window at a
-        // piece's edge may come twice, once without the base beyond the edge,
-        // which adds no base to its sides, and counts are not used.
-        const unsigned long long kMergePiece = std::max<unsigned long long>(1024, 16ull * (h->p.k + 1));
+        // one read and contigs can be millions of bases long (pieces of 4 k
+        // bases, at least 256: most contigs are shorter, and a tile of reads takes
+        // as many rounds as its longest; a piece repeats two windows and up to a
+        // third of its bases.  An iteration of 200 Mbases at k = 31 and 33: 20.2 ms
+        // in pieces of 1024 bases, 19.6 of 512, 19.35 of 256, 19.3 of 128).  Each
+        // window and both its extension bases then lie whole in some piece; a
+        // window at a piece's edge may come twice, once without the base beyond the
+        // edge, which adds no base to its sides, and counts are not used.
+        const unsigned long long kMergePiece = std::max<unsigned long long>(256, 4ull * (h->p.k + 1));
         const unsigned long long kLap = h->p.k + 1;
         DevBuf d_pieces, d_psrc, d_pdst, d_cut;
         std::vector<char> h_pieces;
