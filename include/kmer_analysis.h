@@ -296,9 +296,9 @@ typedef struct {
  * device memory (KMER_DEVICE).  The first
  * lookup after a query, when it asks for an eighth of the survivors at most
  * (and there are 2^20 or more), streams the survivors past the given keys
- * (scratch: 16-32 + 8W bytes per key); any other builds an index of the
- * survivors in device memory (4 bytes per slot, 2-4 slots per survivor), which
- * later lookups reuse.
+ * (scratch: 20-36 + 8W bytes per key; a key given many times costs no more
+ * than different ones); any other builds an index of the survivors in device
+ * memory (4 bytes per slot, 2-4 slots per survivor), which later lookups reuse.
  * Synchronous.  Errors: BAD_STATE (no successful query), INVALID_ARG (NULL
  * with n > 0, bad where), OOM, CUDA. */
 int kmer_analysis_lookup(kmer_analysis_t *h, const uint64_t *keys, uint64_t n, kmer_record *out, int where);

@@ -87,33 +87,67 @@ __global__ void __launch_bounds__(256) lookup_kernel(const unsigned long long* _
 // survivors stream past it once: the partitions come out in that order too, so
 // the slots a survivor needs are in L1 or L2.  1 M k-mers among 101 M
 // survivors: 0.77 ms, against 4.0 for the index.
+//
+// A k-mer given many times (in either orientation) takes one slot: the copy
+// that claims it answers for the others, rep[i] names it, and a last pass
+// hands its record on.  With a slot for every copy, m copies would probe past
+// each other m^2 / 2 times and leave one run of m slots in the way of every
+// survivor that starts in it.
+
+// The canonical form of a given k-mer; returns whether it is the reverse complement.
+template <int W>
+__device__ __forceinline__ bool canonical_of(const unsigned long long* __restrict__ q, unsigned long long i, unsigned k,
+                                             unsigned long long (&key)[W]) {
+    unsigned long long rc[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) key[w] = q[i * W + w];
+    reverse_complement<W>(key, k, rc);
+    const bool flip = key_less<W>(rc, key);
+#pragma unroll
+    for (int w = 0; w < W; ++w) key[w] = flip ? rc[w] : key[w];
+    return flip;
+}
+
 template <int W>
 __global__ void __launch_bounds__(256) wanted_build_kernel(const unsigned long long* __restrict__ q,
                                                            unsigned long long n, const unsigned k,
                                                            unsigned long long* __restrict__ canon,
                                                            unsigned long long* table, unsigned long long cap,
-                                                           kmer_record* __restrict__ out) {
+                                                           unsigned* __restrict__ rep, kmer_record* __restrict__ out) {
     const unsigned hb = 2 * k - 64 * (W - 1), sh = __clzll((long long)cap) + 1;
     for (unsigned long long i = blockIdx.x * 256ull + threadIdx.x; i < n; i += (unsigned long long)gridDim.x * 256) {
-        unsigned long long key[W], rc[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) key[w] = q[i * W + w];
         kmer_record r{};
-        if (key[0] >> hb == 0ull) {  // no bits above 2k (hb is below 64 for odd k)
-            reverse_complement<W>(key, k, rc);
-            const bool flip = key_less<W>(rc, key);
+        unsigned mine = (unsigned)i;
+        if (q[i * W] >> hb == 0ull) {  // no bits above 2k (hb is below 64 for odd k)
+            unsigned long long key[W];
+            r.flipped = canonical_of<W>(q, i, k, key) ? 1 : 0;
 #pragma unroll
-            for (int w = 0; w < W; ++w) canon[i * W + w] = key[w] = flip ? rc[w] : key[w];
-            r.flipped = flip ? 1 : 0;
+            for (int w = 0; w < W; ++w) canon[i * W + w] = key[w];
             const unsigned long long z = aligned_z<W>(key, k);
             const unsigned long long word = (mix_z(z) >> 32) << 32 | (unsigned)(i + 1);
             unsigned long long s = z >> sh;
-            // k-mers given twice take a slot each
+            // slots fill and never empty, so copies of a k-mer meet in the first
+            // slot of its sequence that any of them claims
             for (unsigned long long probe = 0; probe < cap; ++probe) {
-                if (atomicCAS(table + s, 0ull, word) == 0ull) break;
+                unsigned long long e = *(volatile unsigned long long*)(table + s);
+                if (e == 0ull) e = atomicCAS(table + s, 0ull, word);
+                if (e == 0ull) break;  // claimed
+                if ((e ^ word) >> 32 == 0ull) {
+                    unsigned long long other[W];
+                    const unsigned j = (unsigned)e - 1u;
+                    canonical_of<W>(q, j, k, other);
+                    bool same = true;
+#pragma unroll
+                    for (int w = 0; w < W; ++w) same = same && other[w] == key[w];
+                    if (same) {
+                        mine = j;
+                        break;
+                    }
+                }
                 s = (s + 1) & (cap - 1);
             }
         }
+        rep[i] = mine;
         out[i] = r;  // not found, until a survivor says otherwise
     }
 }
@@ -167,6 +201,18 @@ __global__ void __launch_bounds__(256) wanted_stream_kernel(const unsigned long 
                 e[u] = table[s];
             }
         }
+    }
+}
+
+// The records of k-mers given before: the first one's, each with its own `flipped`.
+__global__ void __launch_bounds__(256) wanted_repeat_kernel(const unsigned* __restrict__ rep, unsigned long long n,
+                                                            kmer_record* out) {
+    for (unsigned long long i = blockIdx.x * 256ull + threadIdx.x; i < n; i += (unsigned long long)gridDim.x * 256) {
+        const unsigned j = rep[i];
+        if (j == (unsigned)i) continue;
+        kmer_record r = out[j];
+        r.flipped = out[i].flipped;
+        out[i] = r;
     }
 }
 
@@ -353,26 +399,31 @@ cudaError_t launch_merge_append(unsigned W, const unsigned long long* bkeys, con
     return cudaGetLastError();
 }
 
-size_t wanted_scratch_bytes(unsigned W, unsigned long long n) {
+static unsigned long long wanted_slots(unsigned long long n) {
     unsigned long long cap = 1024;
     while (cap < 2 * n) cap <<= 1;
-    return cap * 8 + n * 8 * W;
+    return cap;
 }
+
+// The table, the canonical k-mers and who answers for each.
+size_t wanted_scratch_bytes(unsigned W, unsigned long long n) { return wanted_slots(n) * 8 + n * 8 * W + n * 4; }
 
 template <int W>
 static cudaError_t launch_wanted_w(const unsigned long long* q, unsigned long long n, unsigned k, void* scratch,
                                    const unsigned long long* keys, const unsigned* count, const unsigned* ext,
                                    const unsigned char* cls, unsigned long long n_out, kmer_record* out, int num_sms,
                                    cudaStream_t s) {
-    const unsigned long long cap = (wanted_scratch_bytes(W, n) - n * 8 * W) / 8;
+    const unsigned long long cap = wanted_slots(n);
     unsigned long long* table = static_cast<unsigned long long*>(scratch);
     unsigned long long* canon = table + cap;
+    unsigned* rep = reinterpret_cast<unsigned*>(canon + n * W);
     cudaError_t e = cudaMemsetAsync(table, 0, cap * 8, s);
     if (e != cudaSuccess) return e;
-    wanted_build_kernel<W><<<grid_of(n, num_sms), 256, 0, s>>>(q, n, k, canon, table, cap, out);
+    wanted_build_kernel<W><<<grid_of(n, num_sms), 256, 0, s>>>(q, n, k, canon, table, cap, rep, out);
     if (n_out)
         wanted_stream_kernel<W><<<grid_of((n_out + 3) / 4, num_sms), 256, 0, s>>>(keys, n_out, k, canon, table, cap,
                                                                                   count, ext, cls, out);
+    wanted_repeat_kernel<<<grid_of(n, num_sms), 256, 0, s>>>(rep, n, out);
     return cudaGetLastError();
 }
 
