@@ -749,6 +749,9 @@ __global__ void __launch_bounds__(kLeafThreads, 2) leaf_kernel(const Job* __rest
                     }
                 }
             }
+            // every warp has read the flags before thread 0 clears them below: one that
+            // came late would sweep a table that is only partly counted
+            __syncthreads();
             clear_table<W>(t, cap);  // leave the table clean
         } else {
             if (threadIdx.x == 0) windows += n;
