@@ -149,6 +149,14 @@ __device__ __forceinline__ uint4 lds128(unsigned a) {
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(a) : "memory");
     return r;
 }
+// The keys of a probe group, which other warps may be claiming: two whole
+// 64-bit words (a vector of 32-bit words would promise nothing about the halves
+// of a tail), split in registers.
+__device__ __forceinline__ uint4 lds_keys(unsigned a) {
+    unsigned long long lo, hi;
+    asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "r"(a) : "memory");
+    return make_uint4((unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32));
+}
 __device__ __forceinline__ void sts32(unsigned a, unsigned v) {
     asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
@@ -250,7 +258,7 @@ __device__ __forceinline__ void probe_round(const Table& t, const unsigned long 
     bool again = false;
     if (have) {
         const unsigned ga = t.tail + 16 * g;
-        const uint4 a = lds128(ga);
+        const uint4 a = lds_keys(ga);
         const bool e0 = same_tail(a.x, a.y, klo, khi), e1 = same_tail(a.z, a.w, klo, khi);
         bool hit = e0 || e1;
         unsigned slot = 2 * g + (e1 ? 1u : 0u);
@@ -310,7 +318,7 @@ __device__ __forceinline__ int find_slot(const Table& t, const unsigned long lon
     unsigned g = __umulhi(hsh, ngroups);
     for (unsigned it = 0; it < kMaxRounds;) {
         const unsigned ga = t.tail + 16 * g;
-        const uint4 a = lds128(ga);
+        const uint4 a = lds_keys(ga);
         if constexpr (W == 2) {
             unsigned long long ct = (unsigned long long)a.y << 32 | a.x, ch = (unsigned long long)a.w << 32 | a.z;
             if (a.x == 0u) {  // empty, or still being claimed
