@@ -224,9 +224,11 @@ struct kmer_analysis {
     double l1_imbalance = 0.0;
     std::vector<unsigned long long> l1_prev_fill;
     unsigned long long l1_prev_windows = 0;
-    // device memory found free by the last query that asked, and its windows
+    // device memory found free by the last query that asked (0: the next one asks),
+    // its windows, and whether the current query plans with it without asking again
     size_t plan_budget = 0;
     unsigned long long plan_windows = 0;
+    bool plan_kept = false;
     kmer_analysis_stats st{};
 
     unsigned W() const { return (2 * p.k + 63) / 64; }
@@ -787,6 +789,10 @@ int run_level2(kmer_analysis* h, Job j, unsigned b0, unsigned nb, unsigned long 
     }
 }
 
+// Internal: the query does not fit the free memory of an earlier moment in one
+// pass without waves, and has to ask for today's first (do_query).
+constexpr int kAskAgain = 1;
+
 // One pass of the partitioned variant over every submitted readset: the
 // scatter, then the level-2 stages over all level-1 buckets at once, or in
 // waves of buckets when their level-2 records do not fit the budget together.
@@ -831,6 +837,7 @@ int run_pass(kmer_analysis* h, const Plan& pl, unsigned pass, unsigned cap_max) 
         const size_t l1_bytes = (size_t)l1_total * 8 * W;
         const size_t avail = pl.budget > l1_bytes ? pl.budget - l1_bytes : 0;
         const bool waves = g.p2 && P1 > 1 && (size_t)l2_full * 8 * W > avail;
+        if (waves && h->plan_kept) return kAskAgain;
         if (h->fb_cap < 64) {
             TRY(h->fb_list.ensure(64 * 4));
             h->fb_cap = 64;
@@ -1112,8 +1119,9 @@ int sort_results(kmer_analysis* h) {
     return KMER_OK;
 }
 
-int do_query(kmer_analysis* h) {
-    const auto t0 = std::chrono::steady_clock::now();
+// One attempt at a query.  `ask`: ask for the free memory also when an answer
+// for this size is kept.
+int query_once(kmer_analysis* h, bool ask) {
     h->have_result = false;
     h->have_contigs = false;
     h->lk_cap = 0;
@@ -1122,6 +1130,7 @@ int do_query(kmer_analysis* h) {
     const kmer_analysis_stats zero{};
     h->st = zero;
     h->st.variant = h->p.variant;
+    h->plan_kept = false;
     unsigned long long windows = 0;
     for (const kmer_readset* rs : h->submitted) windows += rs->windows_for(h->p.k);
     if (windows > 0) {
@@ -1134,8 +1143,11 @@ int do_query(kmer_analysis* h) {
             size_t budget = h->p.memory_budget;
             if (!budget) {
                 // asking for the free memory takes the driver 26 us: a query of about the
-                // last one's size (whose buffers are still here) plans with the last answer
-                if (!h->plan_budget || windows > h->plan_windows || windows < h->plan_windows - h->plan_windows / 8) {
+                // last one's size (whose buffers are still here) plans with the last answer,
+                // unless it needs passes, waves or memory that is gone (do_query)
+                h->plan_kept = !ask && h->plan_budget && windows <= h->plan_windows &&
+                               windows >= h->plan_windows - h->plan_windows / 8;
+                if (!h->plan_kept) {
                     h->plan_budget = (size_t)(0.85 * (double)(free_device_bytes() + h->device_bytes()));
                     h->plan_windows = windows;
                 }
@@ -1170,6 +1182,7 @@ int do_query(kmer_analysis* h) {
                 rec_budget = rec_budget > 2 * fb ? rec_budget - fb : rec_budget / 2;
             }
             const Plan pl = make_plan(h, rec_windows, rec_budget, cap_max, gated_distinct);
+            if (pl.passes > 1 && h->plan_kept) return kAskAgain;
             h->st.pass_bits = pl.g.ps;
             h->st.l1_bits = pl.g.p1;
             h->st.l2_bits = pl.g.p2;
@@ -1193,8 +1206,28 @@ int do_query(kmer_analysis* h) {
     h->st.distinct = h->res_distinct;
     h->st.survivors = h->n_out;
     h->st.device_bytes = h->device_bytes();
-    h->st.ms_total = std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count();
     h->have_result = true;
+    return KMER_OK;
+}
+
+// A query.  One planned with the free memory of an earlier moment runs again
+// with today's when it would take passes or waves (there may be more by now) or
+// finds no memory (there may be less); after passes, waves or an error nothing
+// is kept, so a plan is never the worse for an old answer.
+int do_query(kmer_analysis* h) {
+    const auto t0 = std::chrono::steady_clock::now();
+    int rc = query_once(h, false);
+    if (h->plan_kept && (rc == kAskAgain || rc == KMER_ERR_OOM)) {
+        CK(cudaStreamSynchronize(h->stream));  // the first attempt is done with the pinned counters
+        rc = query_once(h, true);
+    }
+    if (rc != KMER_OK || h->st.passes > 1 || h->st.l2_waves) h->plan_budget = 0;
+    if (rc != KMER_OK) {
+        h->have_result = false;
+        cudaGetLastError();
+        return rc;
+    }
+    h->st.ms_total = std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count();
     return KMER_OK;
 }
 
@@ -1354,13 +1387,7 @@ int kmer_analysis_query(kmer_analysis_t* h, kmer_result_view* out) {
     DeviceGuard dg(h->device);
     StreamScope scope(h->stream);
     std::memset(out, 0, sizeof *out);
-    int rc = do_query(h);
-    if (rc != KMER_OK) {
-        h->have_result = false;
-        h->plan_budget = 0;
-        cudaGetLastError();
-        return rc;
-    }
+    TRY(do_query(h));
     out->n = h->n_out;
     out->k = h->p.k;
     out->words = h->W();
@@ -1384,13 +1411,7 @@ int kmer_analysis_query_into(kmer_analysis_t* h, uint64_t* keys, uint32_t* count
     // own device buffers, then the copy engines (also for sorted output to
     // page-locked arrays: the sort runs in device memory)
     if (where == KMER_HOST_STAGED || (where == KMER_HOST && (h->p.flags & KMER_FLAG_SORTED_OUTPUT))) {
-        const int rc = do_query(h);
-        if (rc != KMER_OK) {
-            h->have_result = false;
-            h->plan_budget = 0;
-            cudaGetLastError();
-            return rc;
-        }
+        TRY(do_query(h));
         if (h->n_out > capacity)
             return fail(KMER_ERR_INVALID_ARG, "%llu survivors do not fit capacity %llu", h->n_out,
                         (unsigned long long)capacity);
@@ -1433,12 +1454,7 @@ int kmer_analysis_query_into(kmer_analysis_t* h, uint64_t* keys, uint32_t* count
     const int rc = do_query(h);
     h->ext_out = false;
     h->out_cap = own_cap;
-    if (rc != KMER_OK) {
-        h->have_result = false;
-        h->plan_budget = 0;
-        cudaGetLastError();
-        return rc;
-    }
+    if (rc != KMER_OK) return rc;
     out->n = h->n_out;
     out->k = h->p.k;
     out->words = h->W();
