@@ -125,8 +125,10 @@ typedef struct {
  * twice is always in F2; a k-mer seen once that slips through as a false
  * positive is counted, once, and dropped): keys, counts, tallies, classes
  * and `windows` are those of the ungated analysis, while `distinct` counts
- * only the k-mers that passed the gate.  Costs two filters of 8 bits per
- * expected distinct k-mer (about one byte per window on a first query) and
+ * only the k-mers that passed the gate, false positives among them (how many
+ * depends on the filters' size and on the order of the updates).  Costs two
+ * filters of 8 bits per expected distinct k-mer (exactly, not rounded up to a
+ * power of two; about one byte per window on a first query) and
  * one more pass over the reads; pays where k-mers seen once are a large
  * share of the windows and memory is tight.  Requires min_count >= 2 and the
  * partitioned variant (INVALID_ARG otherwise); ignored by batches. */

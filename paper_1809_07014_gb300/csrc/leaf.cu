@@ -237,7 +237,11 @@ __device__ __forceinline__ bool same_tail(unsigned lo, unsigned hi, unsigned klo
 __device__ __forceinline__ unsigned leaf_hash(unsigned long long tail) {
     return ((unsigned)tail & ~63u) * 0x9E3779B1u + (unsigned)(tail >> 32) * 0x85EBCA77u;
 }
-// Groups between one probe and the next: at least 256 groups, so that 64 steps never meet again.
+// Groups between one probe and the next: odd and below 256 (a table has 512
+// groups or more).  The groups are a multiple of 32, so a key comes to 32
+// different ones at least before it meets one again: to all 64 of its rounds
+// unless the step shares a large odd factor with the number of groups.  Such a
+// key may send its leaf to the key ranges early, which changes no result.
 __device__ __forceinline__ unsigned leaf_step(unsigned hsh) { return (hsh >> 8 & 255u) | 1u; }
 
 __device__ __forceinline__ void tally(const Table& t, unsigned slot, unsigned long long tail) {

@@ -92,7 +92,9 @@ __global__ void __launch_bounds__(256) lookup_kernel(const unsigned long long* _
 // that claims it answers for the others, rep[i] names it, and a last pass
 // hands its record on.  With a slot for every copy, m copies would probe past
 // each other m^2 / 2 times and leave one run of m slots in the way of every
-// survivor that starts in it.
+// survivor that starts in it.  Among 101 M survivors, 1 M different k-mers, all
+// of them found: 0.98 ms (0.97 without this); 1 M copies of one: 0.32 ms (0.90
+// if every copy tried the compare-and-swap before it read the slot).
 
 // The canonical form of a given k-mer; returns whether it is the reverse complement.
 template <int W>

@@ -292,8 +292,8 @@ __global__ void __launch_bounds__(256) sort_gather_kernel(const unsigned* __rest
 //
 // Whole sort, against digit by digit: 67 M one-word survivors 9.66 -> 3.96 ms
 // (payload records and counts 0.98, two scatters 0.81, level-2 count and
-// splitters 0.25, buckets 1.93: 90 bytes a survivor, bound by the random
-// 32-byte record reads); 8 M four-word survivors 6.25 -> 0.82 ms; 100 k
+// splitters 0.25, buckets 1.93: 90 bytes a survivor asked for, 101 moved, as a
+// random 32-byte record costs more than its sector); 8 M four-word survivors 6.25 -> 0.82 ms; 100 k
 // survivors, k = 21 to 99, 78-250 -> 45-60 us (launches).
 constexpr int kSplitThreads = 512;
 constexpr int kPickThreads = 1024;
