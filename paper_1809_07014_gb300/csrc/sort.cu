@@ -418,16 +418,19 @@ __device__ __forceinline__ unsigned span_shift(unsigned long long span) {
     return sh > 0 ? (unsigned)sh : 0u;
 }
 
-// Exclusive scan of kLut counters in shared memory by a CTA of NT threads.
+// Exclusive scan of kLut counters in shared memory by a CTA of NT threads;
+// returns whether a counter is above `crowd`.
 template <unsigned NT>
-__device__ __forceinline__ void scan_ranges(unsigned* bin, unsigned total, unsigned* warp_tot) {
+__device__ __forceinline__ bool scan_ranges(unsigned* bin, unsigned total, unsigned* warp_tot, unsigned crowd) {
     constexpr unsigned PER = kLut / NT;
     static_assert(PER * NT == kLut, "whole runs");
     unsigned v[PER], sum = 0;
+    bool far = false;
 #pragma unroll
     for (unsigned i = 0; i < PER; ++i) {
         v[i] = bin[threadIdx.x * PER + i];
         sum += v[i];
+        far = far || v[i] > crowd;
     }
     unsigned run = block_scan<NT>(sum, warp_tot);
 #pragma unroll
@@ -436,7 +439,38 @@ __device__ __forceinline__ void scan_ranges(unsigned* bin, unsigned total, unsig
         run += v[i];
     }
     if (threadIdx.x == 0) bin[kLut] = total;
-    __syncthreads();
+    return __syncthreads_or(far);
+}
+
+// Elements 0 .. m - 1 of a CTA's shared memory into ascending order by a bitonic
+// network whose comparators all point up (the places past m stand for elements
+// larger than any and never move): log^2 steps whatever the keys.  The
+// counting within a range takes as many steps as the range has elements, and
+// keys alike in their first bits (error variants of a deep k-mer, amplicons)
+// crowd one range, so a CTA with more than crowd_of elements in some range takes
+// this way.  4 M survivors in clusters of 10 / 50 / 400 that begin with the same
+// 32 bases (16 at k = 31), ms by counting -> as chosen here; random ones; the
+// sort by digits:
+//   k = 31  0.31 / 0.39 / 1.11 -> 0.31 / 0.39 / 0.53;  0.29;  0.6
+//   k = 55  0.61 / 1.32 / 6.49 -> 0.61 / 0.69 / 0.75;  0.38;  1.0
+//   k = 99  0.74 / 1.56 / 7.38 -> 0.72 / 0.75 / 0.81;  0.44;  3.1
+// The lines lie where the two meet: when counting, equal prefixes of two words
+// and more are compared by whole keys in global memory.
+template <int W>
+__device__ __forceinline__ constexpr unsigned crowd_of() { return W >= 2 ? 32 : 128; }
+template <unsigned NT, class Less, class Swap>
+__device__ __forceinline__ void sort_crowded(unsigned m, Less less, Swap swap) {
+    for (unsigned size = 2; size < 2 * m; size <<= 1) {
+        for (unsigned stride = size >> 1; stride; stride >>= 1) {
+            for (unsigned t = threadIdx.x;; t += NT) {
+                const unsigned low = t & (stride - 1), i = (t - low) << 1 | low;  // bit `stride` clear
+                if (i >= m) break;
+                const unsigned j = stride == size >> 1 ? i ^ (size - 1) : i | stride;
+                if (j < m && less(j, i)) swap(i, j);
+            }
+            __syncthreads();
+        }
+    }
 }
 
 // One CTA per group: `over` samples per bucket, ordered in shared memory (as
@@ -482,19 +516,30 @@ __global__ void __launch_bounds__(kPickThreads) split_pick_kernel(const unsigned
             br[u] = b | atomicAdd(&bin[b], 1u) << 16;
         }
     __syncthreads();
-    scan_ranges<kPickThreads>(bin, S, warp_tot);
+    const bool crowded = scan_ranges<kPickThreads>(bin, S, warp_tot, crowd_of<1>());
 #pragma unroll
     for (unsigned u = 0; u < ITEMS; ++u)
         if (u * kPickThreads + threadIdx.x < S) smp[bin[br[u] & 0xFFFFu] + (br[u] >> 16)] = v[u];
     __syncthreads();
+    if (crowded) {
+        sort_crowded<kPickThreads>(
+            S, [&](unsigned x, unsigned y) { return smp[x] < smp[y]; },
+            [&](unsigned x, unsigned y) {
+                const unsigned long long a = smp[x];
+                smp[x] = smp[y];
+                smp[y] = a;
+            });
+        for (unsigned i = threadIdx.x; i + 1 < nb; i += kPickThreads) t.spl[i] = smp[(i + 1) * over];
+    } else {
 #pragma unroll
-    for (unsigned u = 0; u < ITEMS; ++u)
-        if (u * kPickThreads + threadIdx.x < S) {
-            const unsigned b = br[u] & 0xFFFFu, b0 = bin[b], b1 = bin[b + 1], me = b0 + (br[u] >> 16);
-            unsigned f = b0;
-            for (unsigned j = b0; j < b1; ++j) f += smp[j] < v[u] || (smp[j] == v[u] && j < me) ? 1u : 0u;
-            if (f % over == 0 && f) t.spl[f / over - 1] = v[u];
-        }
+        for (unsigned u = 0; u < ITEMS; ++u)
+            if (u * kPickThreads + threadIdx.x < S) {
+                const unsigned b = br[u] & 0xFFFFu, b0 = bin[b], b1 = bin[b + 1], me = b0 + (br[u] >> 16);
+                unsigned f = b0;
+                for (unsigned j = b0; j < b1; ++j) f += smp[j] < v[u] || (smp[j] == v[u] && j < me) ? 1u : 0u;
+                if (f % over == 0 && f) t.spl[f / over - 1] = v[u];
+            }
+    }
     // splitters in ranges before r: those of rank over, 2 over, ... below bin[r]
     for (unsigned r = threadIdx.x; r <= kLut; r += kPickThreads)
         t.first[r] = (unsigned short)(bin[r] ? (bin[r] - 1) / over : 0u);
@@ -714,10 +759,62 @@ __global__ void __launch_bounds__(kSplitThreads, 3) sort_scatter_kernel(
     }
 }
 
+// Survivor x before y by the words after their first 64 bits, which are equal.
+template <int W>
+__device__ __forceinline__ bool tail_less(const unsigned long long* __restrict__ keys, unsigned x, unsigned y) {
+    const unsigned long long *a = keys + (size_t)x * W, *b = keys + (size_t)y * W;
+#pragma unroll
+    for (int w = 1; w < W; ++w)
+        if (a[w] != b[w]) return a[w] < b[w];
+    return false;
+}
+
+// A bucket with a crowded range (not inlined: its registers would cost the
+// ordinary buckets theirs).  `more` (the ranges' counters, no longer used) holds
+// 32 bits after the first 64 of a key where the bucket's elements have room
+// there, so that most comparisons of alike keys stay in shared memory.
+template <int W>
+__device__ __noinline__ void sort_bucket_crowded(unsigned long long* sp, unsigned* si, unsigned* more, unsigned m,
+                                                 unsigned hb, const unsigned long long* __restrict__ kcopy) {
+    const bool wide = W >= 2 && m <= kLut;
+    if constexpr (W >= 2) {
+        if (wide)
+            for (unsigned i = threadIdx.x; i < m; i += kSplitThreads) {
+                const unsigned long long* a = kcopy + (size_t)si[i] * W;
+                unsigned long long x = a[1] << (64 - hb);
+                if constexpr (W >= 3) x |= a[2] >> hb;
+                more[i] = (unsigned)(x >> 32);
+            }
+        __syncthreads();
+    }
+    sort_crowded<kSplitThreads>(
+        m,
+        [&](unsigned x, unsigned y) {
+            const unsigned long long a = sp[x], b = sp[y];
+            if (W == 1 || a != b) return a < b;
+            if (wide && more[x] != more[y]) return more[x] < more[y];
+            return tail_less<W>(kcopy, si[x], si[y]);
+        },
+        [&](unsigned x, unsigned y) {
+            const unsigned long long a = sp[x];
+            const unsigned c = si[x];
+            sp[x] = sp[y];
+            si[x] = si[y];
+            sp[y] = a;
+            si[y] = c;
+            if (wide) {
+                const unsigned d = more[x];
+                more[x] = more[y];
+                more[y] = d;
+            }
+        });
+}
+
 // One CTA per bucket.  The elements are spread over kLut ranges of the
 // bucket's span of prefixes (about one element a range) and ordered within
-// their range by counting the smaller ones; equal prefixes (two words and
-// more) are ordered by their whole keys.  The survivors are then written in
+// their range by counting the smaller ones (a bucket with a crowded range:
+// sort_crowded); equal prefixes (two words and more) are ordered by their whole
+// keys.  The survivors are then written in
 // order: the key (from the prefix, or from the copy of the keys) and the
 // payload record, one random 32-byte read each.  src null: the one bucket of
 // all n keys.
@@ -761,45 +858,49 @@ __global__ void __launch_bounds__(kSplitThreads, 3) sort_buckets_kernel(
             br[u] = b | atomicAdd(&bin[b], 1u) << 16;
         }
     __syncthreads();
-    scan_ranges<kSplitThreads>(bin, m, warp_tot);
+    const bool crowded = scan_ranges<kSplitThreads>(bin, m, warp_tot, crowd_of<W>());
 #pragma unroll
     for (unsigned u = 0; u < kBucketItems; ++u)
         if (u * kSplitThreads + threadIdx.x < m) {
             const unsigned at = bin[br[u] & 0xFFFFu] + (br[u] >> 16);
             sp[at] = p[u];
-            if (W >= 2) si[at] = q[u];
+            if (W >= 2 || crowded) si[at] = q[u];
         }
     __syncthreads();
+    if (crowded) {
+        sort_bucket_crowded<W>(sp, si, bin, m, hb, kcopy);
+    } else {
 #pragma unroll
-    for (unsigned u = 0; u < kBucketItems; ++u)
-        if (u * kSplitThreads + threadIdx.x < m) {
-            const unsigned b = br[u] & 0xFFFFu, b0 = bin[b], b1 = bin[b + 1], me = b0 + (br[u] >> 16);
-            unsigned f = b0;
-            if (b1 - b0 > 1)
-                for (unsigned j = b0; j < b1; ++j) {
-                    const unsigned long long o = sp[j];
-                    bool less = o < p[u];
-                    if (W >= 2 && o == p[u] && j != me) {  // whole keys (their first 64 bits are equal)
-                        const unsigned long long *x = kcopy + (size_t)si[j] * W, *y = kcopy + (size_t)q[u] * W;
+        for (unsigned u = 0; u < kBucketItems; ++u)
+            if (u * kSplitThreads + threadIdx.x < m) {
+                const unsigned b = br[u] & 0xFFFFu, b0 = bin[b], b1 = bin[b + 1], me = b0 + (br[u] >> 16);
+                unsigned f = b0;
+                if (b1 - b0 > 1)
+                    for (unsigned j = b0; j < b1; ++j) {
+                        const unsigned long long o = sp[j];
+                        bool less = o < p[u];
+                        if (W >= 2 && o == p[u] && j != me) {  // whole keys (their first 64 bits are equal)
+                            const unsigned long long *x = kcopy + (size_t)si[j] * W, *y = kcopy + (size_t)q[u] * W;
 #pragma unroll
-                        for (int w = 1; w < W; ++w)
-                            if (x[w] != y[w]) {
-                                less = x[w] < y[w];
-                                break;
-                            }
+                            for (int w = 1; w < W; ++w)
+                                if (x[w] != y[w]) {
+                                    less = x[w] < y[w];
+                                    break;
+                                }
+                        }
+                        f += less ? 1u : 0u;
                     }
-                    f += less ? 1u : 0u;
-                }
-            br[u] = f;
-        }
-    __syncthreads();
+                br[u] = f;
+            }
+        __syncthreads();
 #pragma unroll
-    for (unsigned u = 0; u < kBucketItems; ++u)
-        if (u * kSplitThreads + threadIdx.x < m) {
-            sp[br[u]] = p[u];
-            si[br[u]] = q[u];
-        }
-    __syncthreads();
+        for (unsigned u = 0; u < kBucketItems; ++u)
+            if (u * kSplitThreads + threadIdx.x < m) {
+                sp[br[u]] = p[u];
+                si[br[u]] = q[u];
+            }
+        __syncthreads();
+    }
 #pragma unroll
     for (unsigned u = 0; u < kBucketItems; ++u) {
         const unsigned i = u * kSplitThreads + threadIdx.x;
