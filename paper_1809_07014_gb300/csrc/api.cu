@@ -108,7 +108,8 @@ void pinned_misc_put(Misc* m) {
 }
 
 Geometry plan_geometry(unsigned k, unsigned long long windows, unsigned long long basis, size_t budget,
-                       unsigned cap_max, unsigned leaf_bits, unsigned l1_bits, bool waves, double l1_slack) {
+                       unsigned cap_max, unsigned leaf_bits, unsigned l1_bits, bool waves, double l1_slack,
+                       unsigned fill_bits) {
     Geometry g{};
     g.k = k;
     g.W = (2 * k + 63) / 64;
@@ -122,10 +123,12 @@ Geometry plan_geometry(unsigned k, unsigned long long windows, unsigned long lon
     // ranges)
     const unsigned long long target = std::max(64ull, (unsigned long long)cap_max * 3 / 4);
     unsigned p = leaf_bits ? leaf_bits : ceil_log2((basis + target - 1) / target);
-    // small inputs: a leaf for most CTAs of the leaf kernel (256), of 512 windows
-    // or more (260 000 windows in 64 leaves left four of five CTAs idle)
+    // small inputs: a leaf for most CTAs of the leaf kernel (2^fill_bits; 256 when
+    // the analysis has the launch to itself), of 512 windows or more (260 000
+    // windows in 64 leaves left four of five CTAs idle); and up to 256 leaves while
+    // they have more than 32 768 windows, half of what takes one to the HBM recount
     if (!leaf_bits)
-        while (p < 8 && (windows >> (p + 1)) >= 512) ++p;
+        while (p < 8 && ((windows >> p) > 32768 || (p < fill_bits && (windows >> (p + 1)) >= 512))) ++p;
     const unsigned need = g.bt > 58 ? g.bt - 58 : 0;  // partition bits implied by the record format
     p = std::max(p, need);
     p = std::min(p, g.bt);
